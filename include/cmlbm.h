@@ -208,7 +208,15 @@ int lbm_init_fields_device(lbm_ctx* ctx, const double* phi, const double* p, con
                            const double* uy);
 
 /* Advance nsteps (>= 0) time steps (the update of Secs. 3 - 5 on every node) on params.stream,
- * asynchronous; launch errors are returned.  A run of two or more steps is, where the multi-step
+ * asynchronous; launch errors are returned.  A run of 16 or more steps of a grid whose state the
+ * SMs can hold in shared memory (FP32 arithmetic, up to about 350,000 nodes; the interface
+ * lattice alone up to 650,000; 16-bit storage up to 310,000) is one launch of the resident
+ * kernel: the state is read once, stays on the chip for the run (up to 65536 steps a launch),
+ * and is written back in place.  Its first run allocates the message buffers (up to 30 MB) that
+ * the blocks exchange their borders through; if that fails, in a stream capture, and with a
+ * launch form or shape of the caller's (lbm_set_persistent 0 or 1, lbm_set_graphs 0,
+ * lbm_set_launch) the forms below run instead.
+ * Otherwise a run of two or more steps is, where the multi-step
  * kernel is enabled (lbm_set_persistent; by default with LBM_FP32 storage where the warp
  * segments have at least 3 rows) and the grid's warps fit on the device at once, one launch of
  * that kernel: every warp keeps its strip of columns
@@ -230,10 +238,12 @@ int lbm_set_graphs(lbm_ctx* ctx, int32_t enable);
  * device at once, 0 never, 2 (automatic) where they fit and the warp segments are at least 3
  * rows tall (shorter segments spend more of a step in the waits between steps).  Results are
  * identical.  Default: 2 with LBM_FP32 storage, 0 with the others (where it measured slower
- * than graph replays).  Other values: LBM_ERR_ARG. */
+ * than graph replays).  A call with 0 or 1 also keeps runs from the resident kernel (lbm_step),
+ * a call with 2 allows it again.  Other values: LBM_ERR_ARG. */
 int lbm_set_persistent(lbm_ctx* ctx, int32_t enable);
 
-/* How lbm_step issues a run of two or more steps under the current settings: *path receives
+/* How lbm_step issues a run of two or more steps that the resident kernel does not take (shorter
+ * than 16, or of a grid it cannot hold) under the current settings: *path receives
  * LBM_PATH_MULTI (one multi-step launch), LBM_PATH_GRAPHS (graph replays of one launch per step)
  * or LBM_PATH_SINGLE (one launch per step: graphs off, the bounds-checked kernel, or the first-
  * wait timeout injection).  LBM_ERR_ARG for NULL arguments. */
@@ -310,8 +320,8 @@ int lbm_diagnostics(lbm_ctx* ctx, double xc, double yc, double r_in, double r_ou
 
 /* Tuning of the step launch: rows per warp segment (>= 1) and threads per block (a multiple of
  * 32, 32..256) of the one-launch-per-step kernels; the multi-step kernel takes the segment rows
- * and always runs blocks of 12 warps, one per SM.  0 keeps the current value.  Results do not
- * depend on these. */
+ * and always runs blocks of 12 warps, one per SM.  0 keeps the current value; a value keeps runs
+ * from the resident kernel, whose shape follows from the grid.  Results do not depend on these. */
 int lbm_set_launch(lbm_ctx* ctx, int32_t seg_rows, int32_t block_threads);
 int lbm_get_launch(lbm_ctx* ctx, int32_t* seg_rows, int32_t* block_threads);
 

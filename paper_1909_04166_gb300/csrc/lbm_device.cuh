@@ -18,6 +18,13 @@
 
 namespace cmlbm {
 
+static constexpr unsigned FULL = 0xffffffffu;
+
+// Step variants: bit 0 single relaxation time (Sec. 7) instead of the cascaded rates; bit 1 the
+// interface lattice alone in the imposed shear flow (Sec. 6.1); bit 2 the Langmuir isotherm
+// (Sec. 6.7) instead of the linear sigma(T).
+enum : int { kVarSRT = 1, kVarShear = 2, kVarLangmuir = 4 };
+
 // Per-case constants in the compute precision R.  Derived on the host from lbm_params.
 template <typename R>
 struct Consts {
@@ -124,6 +131,27 @@ struct Geometry {
     int slip;            // free-slip sides: bit 0 left, 1 right, 2 bottom, 3 top
 };
 
+__device__ __forceinline__ int map_row(int y, const Geometry& G)
+{
+    if (y < 0) return G.wall_y ? 0 : y + G.ny;
+    if (y >= G.ny) return G.wall_y ? G.ny - 1 : y - G.ny;
+    return y;
+}
+
+__device__ __forceinline__ int map_col(int x, const Geometry& G)
+{
+    if (x < 0) return G.wall_x ? 0 : x + G.nx;
+    if (x >= G.nx) return G.wall_x ? G.nx - 1 : x - G.nx;
+    return x;
+}
+
+__device__ __forceinline__ unsigned long long global_ns()
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
 // One case of a batch: its geometry and constants, the element offsets of its two state
 // buffers inside the batch allocation, and its warp segmentation.
 template <typename R>
@@ -157,17 +185,33 @@ __device__ __forceinline__ F2 operator-(F2 a, F2 b)
 }
 __device__ __forceinline__ F2& operator+=(F2& a, F2 b) { return a = a + b; }
 
+// One node in the roundings of F2: every product and sum rounded by itself unless fmad says
+// otherwise (plain float expressions may be contracted), so that a kernel may update a node alone
+// or in a pair and store the same bits.
+struct F1 {
+    float v;
+    F1() = default;
+    __device__ __forceinline__ F1(float s) : v(s) {}
+};
+__device__ __forceinline__ F1 operator+(F1 a, F1 b) { return F1(__fadd_rn(a.v, b.v)); }
+__device__ __forceinline__ F1 operator*(F1 a, F1 b) { return F1(__fmul_rn(a.v, b.v)); }
+__device__ __forceinline__ F1 operator-(F1 a, F1 b) { return F1(__fsub_rn(a.v, b.v)); }
+__device__ __forceinline__ F1& operator+=(F1& a, F1 b) { return a = a + b; }
+
 __device__ __forceinline__ float fmad(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fmad(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ F2 fmad(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v, b.v, c.v)); }
+__device__ __forceinline__ F1 fmad(F1 a, F1 b, F1 c) { return F1(__fmaf_rn(a.v, b.v, c.v)); }
 
 template <typename T> struct ScalarOf { using type = T; };
 template <> struct ScalarOf<F2> { using type = float; };
+template <> struct ScalarOf<F1> { using type = float; };
 template <typename T> using scalar_t = typename ScalarOf<T>::type;
 
 template <typename R> __device__ __forceinline__ R log_(R v) { return log(v); }
 template <> __device__ __forceinline__ float log_<float>(float v) { return logf(v); }
 __device__ __forceinline__ F2 log_(F2 v) { return F2(logf(v.v.x), logf(v.v.y)); }
+__device__ __forceinline__ F1 log_(F1 v) { return F1(logf(v.v)); }
 template <typename R> __device__ __forceinline__ void sincospi_(R v, R* s, R* c)
 {
     sincospi(v, s, c);
@@ -182,6 +226,7 @@ __device__ __forceinline__ F2 rcp_(F2 v)
 {
     return F2(__fdividef(1.0f, v.v.x), __fdividef(1.0f, v.v.y));
 }
+__device__ __forceinline__ F1 rcp_(F1 v) { return F1(__fdividef(1.0f, v.v)); }
 // sqrt(v) for v >= 0: exact in double; v * rsqrt(v) in float (0 for v = 0)
 template <typename R> __device__ __forceinline__ R norm_(R v) { return sqrt(v); }
 template <> __device__ __forceinline__ float norm_<float>(float v)
@@ -192,6 +237,10 @@ __device__ __forceinline__ F2 norm_(F2 v)
 {
     return v * F2(rsqrtf(fmaxf(v.v.x, 1e-37f)), rsqrtf(fmaxf(v.v.y, 1e-37f)));
 }
+__device__ __forceinline__ F1 norm_(F1 v)
+{
+    return v * F1(rsqrtf(fmaxf(v.v, 1e-37f)));
+}
 
 // ---------------------------------------------------------------------------------------------
 // Nine-point stencil window of a nodal field: value at (x + i, y + j), i, j in {-1, 0, 1}.
@@ -200,6 +249,16 @@ template <typename T>
 struct Win {
     T sw, s, se, w, c, e, nw, n, ne;
 };
+
+// Value of a window at offset (dx, dy) in {-1, 0, 1}^2.
+template <typename R>
+__device__ __forceinline__ R win_at(const Win<R>& w, int dx, int dy)
+{
+    const R s = dx < 0 ? w.sw : (dx > 0 ? w.se : w.s);
+    const R c = dx < 0 ? w.w : (dx > 0 ? w.e : w.c);
+    const R n = dx < 0 ? w.nw : (dx > 0 ? w.ne : w.n);
+    return dy < 0 ? s : (dy > 0 ? n : c);
+}
 
 // Second-order isotropic differences on the D2Q9 neighbourhood (Sec. 4, closing remark):
 // grad a = 3 sum_a w_a e_a a(x + e_a) and lap a = 6 sum_a w_a (a(x + e_a) - a(x)), with
@@ -652,6 +711,26 @@ __device__ __forceinline__ void equilibria(R phi, R p, R ux, R uy, R rho, R g[9]
     c[8] = third * third * phi;
     central_to_raw(c, ux, uy, r);
     raw_to_pop(r, f);
+}
+
+// Rounding compensation of the 16-bit forms.  Each node stores its eight moving populations
+// first and keeps the sum of their rounding errors (stored minus exact scaled deviation; the
+// difference of a value and its 16-bit rounding is exact in FP32); its rest population, which
+// lands on the node itself, is stored with that sum subtracted.  The stored populations a node
+// sends out then sum to what it computed up to one 16-bit rounding of the rest population's
+// deviation, which is small (the rest state carries no flux), so the lattice sums (the phase
+// mass of the interface lattice) no longer drift with the rounding of every population.
+//
+// Stored value of a population that lands on a node with zeroth moment z: its scaled deviation
+// (v - w z) s, less adj when ADJ; err receives the stored value's rounding error, scaled.
+template <typename S, bool ADJ, typename R>
+__device__ __forceinline__ S encode_err(R v, R z, R w, R scale, R adj, R& err)
+{
+    R d = fmad(-w, z, v) * scale;
+    if constexpr (ADJ) d = d - adj;
+    const S h = f_to_narrow<S>(float(d));
+    err = R(narrow_to_f(h)) - d;
+    return h;
 }
 
 }  // namespace cmlbm

@@ -40,7 +40,6 @@
 
 namespace cmlbm {
 
-static constexpr unsigned FULL = 0xffffffffu;
 static constexpr int TILE = 18 * 32;               // elements per warp-row tile
 static constexpr unsigned WAIT_LIMIT = 1u << 22;   // bounded mbarrier polling (iterations)
 // and in time: a row copy arrives within microseconds, so two seconds of the global timer
@@ -64,11 +63,6 @@ __host__ __device__ inline int flip_of(const void* src, const void* dst)
 {
     return reinterpret_cast<uintptr_t>(src) > reinterpret_cast<uintptr_t>(dst) ? 1 : 0;
 }
-
-// Step variants: bit 0 single relaxation time (Sec. 7) instead of the cascaded rates; bit 1 the
-// interface lattice alone in the imposed shear flow (Sec. 6.1); bit 2 the Langmuir isotherm
-// (Sec. 6.7) instead of the linear sigma(T).
-enum : int { kVarSRT = 1, kVarShear = 2, kVarLangmuir = 4 };
 
 template <typename S> struct Stages { static constexpr int value = 4; };
 template <> struct Stages<double> { static constexpr int value = 3; };
@@ -132,13 +126,6 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
         : "memory");
 }
 
-__device__ __forceinline__ unsigned long long global_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
 // Warp-collective bounded wait for phase `parity` of barrier `bar`; false on timeout (after
 // WAIT_NS of the global timer, or WAIT_LIMIT polls should the timer not advance).  The timer is
 // read only once the first poll has failed, every 64 polls, by lane 0 for the warp.
@@ -170,20 +157,6 @@ template <typename R>
 __device__ __forceinline__ R shfl_up(R v) { return __shfl_up_sync(FULL, v, 1); }
 template <typename R>
 __device__ __forceinline__ R shfl_dn(R v) { return __shfl_down_sync(FULL, v, 1); }
-
-__device__ __forceinline__ int map_row(int y, const Geometry& G)
-{
-    if (y < 0) return G.wall_y ? 0 : y + G.ny;
-    if (y >= G.ny) return G.wall_y ? G.ny - 1 : y - G.ny;
-    return y;
-}
-
-__device__ __forceinline__ int map_col(int x, const Geometry& G)
-{
-    if (x < 0) return G.wall_x ? 0 : x + G.nx;
-    if (x >= G.nx) return G.wall_x ? G.nx - 1 : x - G.nx;
-    return x;
-}
 
 // Element offset of column x (population plane 0) within a row of tiles.
 template <typename S = float>
@@ -323,16 +296,6 @@ __device__ __forceinline__ void st_chk(const BND& B, T* p, T v)
     if (B.wr(p, sizeof(T))) *p = v;
 }
 
-// Value of a window at offset (dx, dy) in {-1, 0, 1}^2.
-template <typename R>
-__device__ __forceinline__ R win_at(const Win<R>& w, int dx, int dy)
-{
-    const R s = dx < 0 ? w.sw : (dx > 0 ? w.se : w.s);
-    const R c = dx < 0 ? w.w : (dx > 0 ? w.e : w.c);
-    const R n = dx < 0 ? w.nw : (dx > 0 ? w.ne : w.n);
-    return dy < 0 ? s : (dy > 0 ? n : c);
-}
-
 // Push the 18 post-collision populations of one node to x + e_a in the row buffers rS, rC, rN
 // (rows y - 1, y, y + 1) at the column offsets cw, cc, ce (columns x - 1, x, x + 1).  fast:
 // warp-uniform, no wall is crossed by any node of this warp row.  Otherwise a population crossing
@@ -380,26 +343,6 @@ __device__ __forceinline__ void push_node(const R g[9], const R f[9], S* rS, S* 
         if (!F_ONLY) st_chk(B, &q[plane * 32], static_cast<S>(g[a]));
         st_chk(B, &q[(9 + plane) * 32], static_cast<S>(f[a]));
     }
-}
-
-// Rounding compensation of the 16-bit forms.  Each node stores its eight moving populations
-// first and keeps the sum of their rounding errors (stored minus exact scaled deviation; the
-// difference of a value and its 16-bit rounding is exact in FP32); its rest population, which
-// lands on the node itself, is stored with that sum subtracted.  The stored populations a node
-// sends out then sum to what it computed up to one 16-bit rounding of the rest population's
-// deviation, which is small (the rest state carries no flux), so the lattice sums (the phase
-// mass of the interface lattice) no longer drift with the rounding of every population.
-//
-// Stored value of a population that lands on a node with zeroth moment z: its scaled deviation
-// (v - w z) s, less adj when ADJ; err receives the stored value's rounding error, scaled.
-template <typename S, bool ADJ, typename R>
-__device__ __forceinline__ S encode_err(R v, R z, R w, R scale, R adj, R& err)
-{
-    R d = fmad(-w, z, v) * scale;
-    if constexpr (ADJ) d = d - adj;
-    const S h = f_to_narrow<S>(float(d));
-    err = R(narrow_to_f(h)) - d;
-    return h;
 }
 
 // As push_node for the 16-bit forms: every population is stored as its deviation from the rest

@@ -1203,8 +1203,12 @@ __device__ __forceinline__ void step_body(const S* __restrict__ src, S* __restri
                            L.chk_shrink, cut);
 }
 
+// 168 registers a thread are what 12 resident warps per SM leave (the shared memory of the FP32
+// ring allows no more); the compiler's own choice under __launch_bounds__(256) is 126, a residency
+// it cannot have, and costs more instructions: 393.5 against 387.3 us a step on the 4096 x 4096
+// impact, 54.4 against 53.4 on 2048 x 1024, 21.1 against 20.3 on 1501 x 501 (graph replays).
 template <typename R, typename S, int V>
-__global__ void __launch_bounds__(256)
+__global__ void __maxnreg__(168)
 step_kernel(const S* __restrict__ src, S* __restrict__ dst, Geometry G, Consts<R> K,
             StepLaunch L)
 {

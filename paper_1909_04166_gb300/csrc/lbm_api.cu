@@ -95,8 +95,45 @@ void* cur_state(lbm_ctx* c) { return c->buf + (size_t)c->cur * c->state_bytes; }
 // in two waves; a partial wave is slower than one full wave).
 constexpr int kSegRows = 16;
 
+// FP64: the double-precision unit sets the time.  A double-precision instruction of a warp takes it
+// kDpSm cycles of its SM where four or more warps share the SM, and never less than kDpWarp (both
+// measured, whatever the lanes active), so a step takes what the SM with the most warps needs:
+// the rows of a segment, about kDpRow instructions each, and the sums of the two rows around it
+// (kDpSeg); the fewer warps share the SM, the more of their other latencies shows (kDpFew).  With
+// one-warp blocks the scheduler spreads the warps evenly; warps beyond the resident ones wait for a
+// second wave.  The shortest such time over the segment heights up to kDpMaxRows decides (one GB300, us a step, the former whole-wave rule in 4-warp
+// blocks against this one: 64 x 64 18.0 / 16.5, 256 x 256 57.8 / 50.4, 512 x 256 123 / 94, 700 x
+// 450 238 / 218, 600 x 300 162 / 138).
+constexpr double kDpSm = 19, kDpWarp = 64, kDpRow = 365, kDpSeg = 50, kDpFew = 0.3;
+constexpr int kDpMaxRows = 24;
+
+int fp64_seg_rows(const lbm_ctx* c)
+{
+    const int resident = with_variant(c->P.precision, c->variant, [&](auto r, auto s, auto v) {
+        return step_blocks_per_sm<decltype(r), decltype(s), decltype(v)::value>(c->block) *
+               (c->block / 32);
+    });
+    auto shared = [](long long k) {   // cycles per instruction of each of k warps on an SM
+        return k == 0 ? 0.0 : std::max(kDpWarp, kDpSm * k) * (1 + kDpFew / k);
+    };
+    double best = 0;
+    int best_h = 1;
+    for (int h = 1; h <= kDpMaxRows && h <= c->G.ny; ++h) {
+        const long long warps = (long long)c->G.nstrips * ((c->G.ny + h - 1) / h);
+        const long long per_sm = (warps + c->nsm - 1) / c->nsm;
+        const double t = (h * kDpRow + kDpSeg) *
+                         (per_sm / resident * shared(resident) + shared(per_sm % resident));
+        if (h == 1 || t < best) {
+            best = t;
+            best_h = h;
+        }
+    }
+    return best_h;
+}
+
 int default_seg_rows(const lbm_ctx* c)
 {
+    if (c->P.precision == LBM_FP64) return fp64_seg_rows(c);
     int strips_per_row = 1;
     const int bps = with_variant(c->P.precision, c->variant, [&](auto r, auto s, auto v) {
         using R = decltype(r);
@@ -339,7 +376,7 @@ int make_ctx(const lbm_params* params, void* ext, size_t ext_bytes, lbm_ctx** ou
     int dev = params->device, nsm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     c->nsm = nsm > 0 ? nsm : 1;
-    c->block = 128;
+    c->block = params->precision == LBM_FP64 ? 32 : 128;
     c->use_graph = 1;
     // the multi-step kernel automatically for FP32 storage (measured faster than graph replays
     // there on grids of tall segments; slower with FP64 and 16-bit storage)

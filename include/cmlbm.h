@@ -412,7 +412,13 @@ int lbm_batch_case_transposed(const lbm_batch* b, int32_t c);
 int lbm_batch_init_fields(lbm_batch* b, int32_t c, const double* phi, const double* p,
                           const double* ux, const double* uy);
 
-/* Advance every case by nsteps (>= 0) time steps; asynchronous on the batch's stream. */
+/* Advance every case by nsteps (>= 0) time steps; asynchronous on the batch's stream.  A run of
+ * 16 or more steps (64 with 16-bit storage in large batches) of a batch with FP32 arithmetic whose
+ * cases each fit the SMs' shared memory is issued as one launch of the resident kernel (lbm_step)
+ * per wave, a set of cases that fit together, each launch taking its cases through all the steps;
+ * the first such run allocates the message buffers (about 3 MB a wave).  If that fails, in a stream
+ * capture, and once the caller has chosen a form or shape (lbm_batch_set_persistent,
+ * lbm_batch_set_launch), runs take the other forms.  The results are the same, bit for bit. */
 int lbm_batch_step(lbm_batch* b, int32_t nsteps);
 
 /* Fields / populations of case c, as lbm_get_fields / lbm_get_populations.  Synchronise. */
@@ -420,8 +426,9 @@ int lbm_batch_get_fields(lbm_batch* b, int32_t c, double* phi, double* p, double
                          double* uy, double* rho);
 int lbm_batch_get_populations(lbm_batch* b, int32_t c, double* g, double* f);
 
-/* Launch shape: rows per warp task (>= 1) and threads per block (multiple of 32, <= 256);
- * 0 keeps the current value.  Results do not depend on it. */
+/* Launch shape of the one-launch-per-step kernel: rows per warp task (>= 1) and threads per block
+ * (multiple of 32, <= 256); 0 keeps the current value, a value keeps runs from the resident kernel.
+ * Results do not depend on it. */
 int lbm_batch_set_launch(lbm_batch* b, int32_t seg_rows, int32_t block_threads);
 int lbm_batch_get_launch(const lbm_batch* b, int32_t* seg_rows, int32_t* block_threads);
 
@@ -430,15 +437,18 @@ int lbm_batch_get_launch(const lbm_batch* b, int32_t* seg_rows, int32_t* block_t
  * block per SM, whose warps share the batch's warp tasks out once, balanced by nodes, and take
  * their tasks in a fixed order every step; a task waits, before its step, only for the tasks of
  * the same case within reach of its reads and writes.  enable = 0 (default): graph replays of
- * one launch per step.  The results are the same, bit for bit.  Other values: LBM_ERR_ARG.
- * lbm_batch_get_step_path: LBM_PATH_MULTI where the multi-step kernel takes the runs (enabled,
- * and its warps fit on the device at once), else LBM_PATH_GRAPHS. */
+ * one launch per step.  Either call keeps runs from the resident kernel (lbm_batch_step).  The
+ * results are the same, bit for bit.  Other values: LBM_ERR_ARG.
+ * lbm_batch_get_step_path: LBM_PATH_MULTI where the multi-step kernel takes the runs that the
+ * resident kernel does not (enabled, and its warps fit on the device at once), else
+ * LBM_PATH_GRAPHS. */
 int lbm_batch_set_persistent(lbm_batch* b, int32_t enable);
 int lbm_batch_get_step_path(const lbm_batch* b, int32_t* path);
 
 /* Autotuner: times trial_steps (>= 1) steps of the live batch for each candidate launch shape
  * (rows per task 8..64, blocks of 64 or 128 threads), keeps the fastest and restores the state
- * it started from (a temporary device copy).  Synchronises. */
+ * it started from (a temporary device copy).  Which runs the resident kernel takes stays as it
+ * was.  Synchronises. */
 int lbm_batch_tune(lbm_batch* b, int32_t trial_steps, int32_t* seg_rows, int32_t* block_threads);
 
 /* Total nodes of all cases; LBM_ERR_TIMEOUT check as lbm_check; release (NULL allowed). */

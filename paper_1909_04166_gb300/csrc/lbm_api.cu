@@ -210,7 +210,7 @@ constexpr int kResidentMinSteps = 16;
 
 void* resident_lists(const lbm_ctx* c)
 {
-    return static_cast<char*>(c->box) + c->rplan.box_bytes;
+    return static_cast<char*>(c->box) + c->rplan.Z.box_bytes;
 }
 
 // The resident kernel takes a run: allowed (not with a launch form or shape chosen by the
@@ -238,7 +238,7 @@ bool resident_takes(lbm_ctx* c, long long run)
             else return false;
         });
         if (!ok) return false;
-        const size_t bytes = c->rplan.box_bytes + c->rplan.list_bytes;
+        const size_t bytes = c->rplan.Z.box_bytes + c->rplan.Z.list_bytes;
         if (cudaMalloc(&c->box, bytes) != cudaSuccess) {
             cudaGetLastError();
             c->box = nullptr;

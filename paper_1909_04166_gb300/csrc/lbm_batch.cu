@@ -15,12 +15,14 @@
 #include <algorithm>
 #include <cmath>
 #include <new>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
 #include "../../include/cmlbm.h"
 #include "lbm_device.cuh"
 #include "lbm_host.h"
+#include "lbm_resident.h"
 
 using namespace cmlbm;
 
@@ -90,6 +92,14 @@ struct lbm_batch {
     int* dorder;
     int* dwbeg;
     unsigned* dprog;
+    // the resident kernel (lbm_resident.cu): its waves, and in one allocation their mailboxes,
+    // exchange lists, case descriptors and block tables
+    int use_resident;
+    int resident_state;     // 0: no plan made yet, 1: ready, -1: not usable
+    std::vector<ResidentWave> waves;
+    char* rmem;
+    std::vector<size_t> wave_lists, wave_cases, wave_blocks;   // offsets in rmem
+    unsigned rtag;          // tag of the last message sent
 };
 
 namespace {
@@ -288,6 +298,120 @@ cudaError_t ensure_graphs(lbm_batch* b)
     return e;
 }
 
+// Shortest runs that go to the resident kernel, every wave of which is a launch that reads and
+// writes its part of the state once; 16-bit storage, whose steps gain less, in batches of more
+// than kBatchFewWaves waves only from kBatchResidentMinSteps16Bit on.  One GB300, us a step against
+// graph replays: 192 drops of sides 32 - 256 (18 waves), FP32, 16 steps 131 / 138, 1000 steps 107 /
+// 137; FP16, 32 steps 171 / 156, 64 steps 152 / 156, 1000 steps 143 / 155; 16 such drops (one or
+// two waves) 6.3 / 26 and 8.4 / 36.
+constexpr int kBatchResidentMinSteps = 16, kBatchResidentMinSteps16Bit = 64;
+constexpr size_t kBatchFewWaves = 2;
+
+// Call f(S{}, V{}) for the batch's storage and step variant where the resident kernel has them.
+template <class F>
+bool with_resident(const lbm_batch* b, F&& f)
+{
+    return with_variant(b->precision, b->variant, [&](auto r, auto s, auto v) -> bool {
+        if constexpr (std::is_same<decltype(r), float>::value && (decltype(v)::value & 2) == 0)
+            return f(s, v);
+        else return false;
+    });
+}
+
+// Make the waves, allocate what they need and fill it; false if a case does not fit or the
+// memory is not there.
+bool plan_resident(lbm_batch* b)
+{
+    const int n = (int)b->cases.size();
+    std::vector<Geometry> G;
+    for (const HostCase& hc : b->cases) G.push_back(hc.G);
+    if (!with_resident(b, [&](auto s, auto v) {
+            return resident_batch_plan<decltype(s), decltype(v)::value>(G.data(), n, b->nsm,
+                                                                        &b->waves);
+        })) {
+        b->waves.clear();
+        return false;
+    }
+    size_t bytes = 0, box = 0;
+    auto place = [&](size_t size) {
+        const size_t at = bytes;
+        bytes += (size + 255) / 256 * 256;
+        return at;
+    };
+    for (const ResidentWave& w : b->waves) box = std::max(box, w.Z.box_bytes);
+    place(box);   // the waves run one after another and share the mailboxes
+    b->wave_lists.clear();
+    b->wave_cases.clear();
+    b->wave_blocks.clear();
+    for (const ResidentWave& w : b->waves) {
+        b->wave_lists.push_back(place(w.Z.list_bytes));
+        b->wave_cases.push_back(place(w.cases.size() * sizeof(ResidentCase)));
+        b->wave_blocks.push_back(place(w.Z.nblocks * sizeof(int)));
+    }
+    if (cudaMalloc(&b->rmem, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        b->rmem = nullptr;
+        return false;
+    }
+    cudaError_t e = cudaMemsetAsync(b->rmem, 0, box, b->st);
+    for (size_t k = 0; k < b->waves.size() && e == cudaSuccess; ++k) {
+        const ResidentWave& w = b->waves[k];
+        std::vector<ResidentCase> cases;
+        std::vector<int> block;
+        for (size_t j = 0; j < w.cases.size(); ++j) {
+            const HostCase& hc = b->cases[w.cases[j]];
+            cases.push_back(ResidentCase{hc.G, w.D[j], {hc.off0, hc.off1}, hc.Kf});
+            block.insert(block.end(), w.D[j].nstrip * w.D[j].nseg, (int)j);
+        }
+        auto* dc = reinterpret_cast<ResidentCase*>(b->rmem + b->wave_cases[k]);
+        int* db = reinterpret_cast<int*>(b->rmem + b->wave_blocks[k]);
+        // pageable host memory: both copies have left it when the calls return
+        e = cudaMemcpyAsync(dc, cases.data(), cases.size() * sizeof(ResidentCase),
+                            cudaMemcpyHostToDevice, b->st);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(db, block.data(), block.size() * sizeof(int),
+                                cudaMemcpyHostToDevice, b->st);
+        if (e != cudaSuccess) break;
+        with_resident(b, [&](auto s, auto v) {
+            e = prepare_resident_batch<decltype(s), decltype(v)::value>(
+                w.Z, dc, db, b->rmem + b->wave_lists[k], b->st);
+            return true;
+        });
+    }
+    return e == cudaSuccess;
+}
+
+// The resident kernel takes a run: allowed (no launch form or shape of the caller's), long
+// enough, planned, and outside a stream capture (as in lbm_api.cu).
+bool resident_takes(lbm_batch* b, int run)
+{
+    if (!b->use_resident || b->resident_state < 0 || run < kBatchResidentMinSteps) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(b->st, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (cap != cudaStreamCaptureStatusNone) return false;
+    if (b->resident_state == 0) b->resident_state = plan_resident(b) ? 1 : -1;
+    const bool narrow = b->precision == LBM_FP32_FP16 || b->precision == LBM_FP32_BF16;
+    return b->resident_state == 1 && !(narrow && b->waves.size() > kBatchFewWaves &&
+                                       run < kBatchResidentMinSteps16Bit);
+}
+
+cudaError_t launch_resident_wave(lbm_batch* b, size_t k, int nsteps)
+{
+    cudaError_t e = cudaErrorInvalidValue;
+    with_resident(b, [&](auto s, auto v) {
+        e = launch_resident_batch<decltype(s), decltype(v)::value>(
+            b->base, b->waves[k].Z, reinterpret_cast<ResidentCase*>(b->rmem + b->wave_cases[k]),
+            reinterpret_cast<int*>(b->rmem + b->wave_blocks[k]), b->cur, nsteps, b->rtag, b->rmem,
+            b->rmem + b->wave_lists[k], b->err, b->st);
+        return true;
+    });
+    if (e == cudaSuccess) b->rtag += (unsigned)nsteps;
+    return e;
+}
+
 template <typename R> const Consts<R>& kref(const HostCase& hc);
 template <> const Consts<double>& kref<double>(const HostCase& hc) { return hc.Kd; }
 template <> const Consts<float>& kref<float>(const HostCase& hc) { return hc.Kf; }
@@ -341,6 +465,7 @@ int lbm_batch_create_ex(const lbm_params* params, int32_t ncases, int32_t layout
     b->elem = elem_bytes(b->precision);
     b->st = static_cast<cudaStream_t>(params[0].stream);
     b->block = 128;
+    b->use_resident = 1;
     int nsm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b->device);
     b->nsm = nsm > 0 ? nsm : 1;
@@ -429,6 +554,21 @@ int lbm_batch_step(lbm_batch* b, int32_t nsteps)
     if (!b || nsteps < 0) return LBM_ERR_ARG;
     cudaSetDevice(b->device);
     int32_t k = 0;
+    while (resident_takes(b, nsteps - k)) {   // in place: the parity is unchanged
+        const int chunk = std::min(nsteps - k, 1 << 16);
+        cudaError_t e = cudaSuccess;
+        for (size_t w = 0; w < b->waves.size() && e == cudaSuccess; ++w) {
+            e = launch_resident_wave(b, w, chunk);
+            if (e == cudaErrorCooperativeLaunchTooLarge && w == 0) break;
+            if (e != cudaSuccess) return fail_cuda(b, e);
+        }
+        if (e != cudaSuccess) {   // fewer SMs here than the device has
+            cudaGetLastError();
+            b->resident_state = -1;
+            break;
+        }
+        k += chunk;
+    }
     while (nsteps - k >= 2 && multi_fits(b)) {   // one multi-step launch per 65536 steps
         const int chunk = std::min(nsteps - k, 1 << 16);
         cudaError_t e = launch_multi_run(b, chunk);
@@ -519,6 +659,7 @@ int lbm_batch_set_launch(lbm_batch* b, int32_t seg_rows, int32_t block_threads)
     if (!b || seg_rows < 0 || block_threads < 0) return LBM_ERR_ARG;
     if (block_threads && (block_threads % 32 || block_threads > 256)) return LBM_ERR_ARG;
     cudaSetDevice(b->device);
+    if (seg_rows || block_threads) b->use_resident = 0;   // the caller's shape
     if (block_threads) {
         b->block = block_threads;
         drop_batch_graphs(b);
@@ -532,6 +673,7 @@ int lbm_batch_set_persistent(lbm_batch* b, int32_t enable)
 {
     if (!b || enable < 0 || enable > 1) return LBM_ERR_ARG;
     b->use_multi = enable;
+    b->use_resident = 0;
     return LBM_OK;
 }
 
@@ -563,7 +705,7 @@ int lbm_batch_tune(lbm_batch* b, int32_t trial_steps, int32_t* seg_rows, int32_t
         if (backup) cudaFree(backup);
         return fail_cuda(b, e);
     }
-    const int cur0 = b->cur;
+    const int cur0 = b->cur, resident0 = b->use_resident;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -609,6 +751,7 @@ int lbm_batch_tune(lbm_batch* b, int32_t trial_steps, int32_t* seg_rows, int32_t
     if (e2 != cudaSuccess) return fail_cuda(b, e2);
     if (status) return status;
     status = lbm_batch_set_launch(b, best_seg, best_block);
+    b->use_resident = resident0;   // the tuner's shape is for the runs it does not take
     if (status) return status;
     if (seg_rows) *seg_rows = best_seg;
     if (block_threads) *block_threads = best_block;
@@ -644,6 +787,7 @@ void lbm_batch_destroy(lbm_batch* b)
     if (b->dorder) cudaFree(b->dorder);
     if (b->dwbeg) cudaFree(b->dwbeg);
     if (b->dprog) cudaFree(b->dprog);
+    if (b->rmem) cudaFree(b->rmem);
     delete b;
 }
 

@@ -19,6 +19,9 @@
 // a block sends step t + 2 only after the messages of step t + 1 of all its neighbours have
 // arrived, which those sent after reading step t's.
 //
+// A batch is taken in waves of cases whose blocks fit on the device together, one launch a wave for
+// all the steps of a run: a case's neighbours are its own blocks, so cases never wait for each other.
+//
 // Per node the arithmetic is the paired march's of lbm_step.cu (F2, or F1 with the same
 // roundings), the zeroth moments are summed in its orders (in plane order; in the halo's tree
 // order for the columns next to a strip), and the 16-bit forms round every pushed population as
@@ -40,7 +43,9 @@
 #include "lbm_device.cuh"
 #include "lbm_resident.h"
 
+#include <algorithm>
 #include <type_traits>
+#include <vector>
 
 namespace cmlbm {
 
@@ -211,26 +216,63 @@ __device__ __forceinline__ void ring_node(int j, int h, int w, int& r, int& c)
         c = ci < 2 ? ci - 1 : w + ci - 3;
     }
 }
-__device__ __forceinline__ Block block_of(const Geometry& G, const ResidentLaunch& L)
+__device__ __forceinline__ Block block_of(const Geometry& G, const ResidentGrid& D)
 {
+    const int b = (int)blockIdx.x - D.block0;
     Block B;
-    B.strip = blockIdx.x % L.nstrip;
-    B.seg = blockIdx.x / L.nstrip;
+    B.strip = b % D.nstrip;
+    B.seg = b / D.nstrip;
     B.x0 = B.strip * 64;
     B.w = strip_cols(B.strip, G.nx);
-    B.y0 = seg_start(B.seg, L.nseg, G.ny);
-    B.h = seg_rows_of(B.seg, L.nseg, G.ny);
+    B.y0 = seg_start(B.seg, D.nseg, G.ny);
+    B.h = seg_rows_of(B.seg, D.nseg, G.ny);
     return B;
+}
+
+// A neighbour of a block: dx strips (-2 .. 2) and dy segments (-1 .. 1) away.  The blocks beyond
+// the next strip hold a common node with this one where that strip, the last of the grid, is a
+// single column.
+struct Neighbour {
+    bool exists;
+    int strip, seg;
+    int dc, dr;   // its column 0 and row 0 in this block's coordinates
+};
+__device__ __forceinline__ Neighbour neighbour(const Geometry& G, const Block& B,
+                                               const ResidentGrid& D, int dx, int dy)
+{
+    Neighbour N;
+    N.strip = B.strip + dx;
+    N.seg = B.seg + dy;
+    N.exists = (dx || dy) && !(G.wall_x && (N.strip < 0 || N.strip >= D.nstrip)) &&
+               !(G.wall_y && (N.seg < 0 || N.seg >= D.nseg));
+    N.strip = (N.strip + 2 * D.nstrip) % D.nstrip;
+    N.seg = (N.seg + D.nseg) % D.nseg;
+    const int between = (B.strip + dx / 2 + D.nstrip) % D.nstrip;   // for dx = -2, 2
+    if ((dx == 2 || dx == -2) && strip_cols(between, G.nx) != 1) N.exists = false;
+    N.dc = dx > 0 ? B.w + (dx == 2 ? 1 : 0)
+                  : (dx < 0 ? -strip_cols(N.strip, G.nx) - (dx == -2 ? 1 : 0) : 0);
+    N.dr = dy > 0 ? B.h : (dy < 0 ? -seg_rows_of(N.seg, D.nseg, G.ny) : 0);
+    return N;
+}
+// The imposed-flow form (taller blocks, longer lists) has 13 bits for a mailbox index, and no
+// single-column strips; the others 12.
+template <int V> __host__ __device__ constexpr int reach() { return (V & kVarShear) ? 1 : 2; }
+template <int V> __host__ __device__ constexpr int box_bits() { return (V & kVarShear) ? 13 : 12; }
+template <int V>
+__host__ __device__ constexpr int neighbour_code(int dx, int dy)   // below 1 << (16 - box_bits)
+{
+    const int k = (dy + 1) * (2 * reach<V>() + 1) + dx + reach<V>();
+    return (V & kVarShear) && k > 4 ? k - 1 : k;
 }
 
 // Setup, once per plan: the exchange lists of every block, in the order of the mailbox
 // (consecutive threads take consecutive columns; any order would do), after the numbers of
 // sends and receives.
 template <int V>
-__global__ void __launch_bounds__(NT) resident_lists_kernel(Geometry G, ResidentLaunch L)
+__device__ void build_lists(const Geometry& G, const ResidentGrid& D, const ResidentLaunch& L)
 {
     __shared__ int count[2];
-    const Block B = block_of(G, L);
+    const Block B = block_of(G, D);
     int* out = L.lists + blockIdx.x * (2 + list_words(L.hmax, L.tab));
     const Lists T = lists_at(out + 2, L.hmax, L.tab);
     if (threadIdx.x < 2) count[threadIdx.x] = 0;
@@ -239,7 +281,8 @@ __global__ void __launch_bounds__(NT) resident_lists_kernel(Geometry G, Resident
         int r, c;
         ring_node(j, B.h, B.w, r, c);
         const int gx = B.x0 + c, gy = B.y0 + r - 1;
-        bool ok = c <= B.w;
+        // (a single column of a side row would be there twice)
+        bool ok = c <= B.w && !(B.w == 1 && j >= 4 * RW + 2 * (B.h - 2) && c == 0);
         if (G.wall_x && (gx < 0 || gx >= G.nx)) ok = false;
         if (G.wall_y && (gy < 0 || gy >= G.ny)) ok = false;
         T.node[j] = ok ? (unsigned)r << 16 | (unsigned)(c + 1) : kNoNode;
@@ -285,43 +328,164 @@ __global__ void __launch_bounds__(NT) resident_lists_kernel(Geometry G, Resident
             T.roff[ar] = off;
             T.rbox[ar] = (unsigned short)i;
         }
-        for (int d = 0; d < 9; ++d) {
-            const int dx = d % 3 - 1, dy = d / 3 - 1;
-            if (dx == 0 && dy == 0) continue;
-            bool to = ok && mine;
-            int c2 = c, r2 = r, s2 = B.strip + dx, g2 = B.seg + dy;
-            if (dx > 0) to = to && c >= B.w - 1;
-            if (dx < 0) to = to && c <= 0;
-            if (dy > 0) to = to && r >= B.h;
-            if (dy < 0) to = to && r <= 1;
-            if (s2 < 0 || s2 >= L.nstrip) {
-                if (G.wall_x) to = false;
-                s2 = s2 < 0 ? L.nstrip - 1 : 0;
+        for (int dy = -1; dy <= 1; ++dy)
+            for (int dx = -reach<V>(); dx <= reach<V>(); ++dx) {
+                const Neighbour N = neighbour(G, B, D, dx, dy);
+                const int c2 = c - N.dc, r2 = r - N.dr;
+                const int w2 = strip_cols(N.strip, G.nx), h2 = seg_rows_of(N.seg, D.nseg, G.ny);
+                const int as = append(ok && mine && N.exists && c2 >= -1 && c2 <= w2 && r2 >= 0 &&
+                                          r2 <= h2 + 1,
+                                      0);
+                if (as >= 0) {
+                    T.soff[as] = off;
+                    T.sdst[as] = (unsigned short)(neighbour_code<V>(dx, dy) << box_bits<V>() |
+                                                  box_index(r2, c2, a, h2, w2, L.hmax));
+                }
             }
-            if (g2 < 0 || g2 >= L.nseg) {
-                if (G.wall_y) to = false;
-                g2 = g2 < 0 ? L.nseg - 1 : 0;
-            }
-            const int w2 = strip_cols(s2, G.nx), h2 = seg_rows_of(g2, L.nseg, G.ny);
-            if (dx > 0) c2 -= B.w;
-            if (dx < 0) c2 += w2;
-            if (dy > 0) r2 -= B.h;
-            if (dy < 0) r2 += h2;
-            const int as = append(to, 0);
-            if (as >= 0) {
-                T.soff[as] = off;
-                T.sdst[as] = (unsigned short)((d < 4 ? d : d - 1) << 13 |
-                                              box_index(r2, c2, a, h2, w2, L.hmax));
-            }
-        }
     }
     __syncthreads();
-    if (threadIdx.x < 2) out[threadIdx.x] = min(count[threadIdx.x], L.tab);
+    if (threadIdx.x < 2) out[threadIdx.x] = count[threadIdx.x];
 }
 
+template <int V>
+__global__ void __launch_bounds__(NT) resident_lists_kernel(Geometry G, ResidentGrid D,
+                                                            ResidentLaunch L)
+{
+    build_lists<V>(G, D, L);
+}
+template <int V>
+__global__ void __launch_bounds__(NT)
+resident_batch_lists_kernel(const ResidentCase* __restrict__ cases,
+                            const int* __restrict__ case_of, ResidentLaunch L)
+{
+    const ResidentCase& c = cases[case_of[blockIdx.x]];
+    build_lists<V>(c.G, c.D, L);
+}
+
+// 16-byte accesses to the tiles of a block's rows: flat index -> (row, tile, access) and where its
+// first element sits: plane p and column c (a 16-bit tile starts with its two Z planes, p = -2 and
+// -1, in floats).
+template <typename S, int V>
+struct TileVec {
+    static constexpr bool SHEAR = (V & kVarShear) != 0;
+    static constexpr int TE = Tile<S>::ELEMS;
+    static constexpr int EV = 16 / (int)sizeof(S);             // elements of an access
+    static constexpr int TV0 = SHEAR ? 9 * 32 / EV : 0;        // first one of a tile that is needed
+    static constexpr int TV = TE / EV - TV0;                   // and how many follow
+    struct At { int r, t, q, p, c; };
+    static __device__ __forceinline__ At at(int ntiles, int i)
+    {
+        At a;
+        a.r = i / (ntiles * TV);
+        const int k = i - a.r * (ntiles * TV);
+        a.t = k / TV;
+        a.q = k - a.t * TV + TV0;
+        constexpr int ZV = Tile<S>::ZBYTES / 16;               // 8 accesses a Z plane
+        if (a.q < ZV) {
+            a.p = a.q / 8 - 2;
+            a.c = 32 * a.t + a.q % 8 * 4;
+        } else {
+            a.p = (a.q - ZV) * EV / 32 - (SHEAR ? 9 : 0);
+            a.c = 32 * a.t + (a.q - ZV) * EV % 32;
+        }
+        return a;
+    }
+};
+
+__device__ __forceinline__ bool row_exists(const Geometry& G, const Block& B, int r)
+{
+    const int gy = B.y0 + r - 1;
+    return !(G.wall_y && (gy < 0 || gy >= G.ny));
+}
+template <typename S>
+__device__ __forceinline__ S* global_row(const Geometry& G, const Block& B, S* state, int r)
+{
+    return state + (long long)map_row(B.y0 + r - 1, G) * G.nstrips * Tile<S>::ELEMS;
+}
+
+// Load a block and its ghost ring: the tiles of every row 16 bytes at a time, several loads of a
+// thread in flight, then the two ghost columns.  (Not inlined: the registers of the time loop.)
+template <typename S, int V>
+__device__ __noinline__ void load_block(S* state, Geometry G, Block B, float* pop, float* sps,
+                                        float* sph, float* gz)
+{
+    using VA = TileVec<S, V>;
+    constexpr bool SHEAR = VA::SHEAR, NARROW = Narrow<S>::value;
+    constexpr int PL = SHEAR ? 9 : 18, ROWF = row_floats<V>();
+    const int tid = threadIdx.x, h = B.h, w = B.w, ntiles = (w + 31) / 32;
+    {
+        constexpr int U = 4;
+        const int total = (h + 2) * ntiles * VA::TV;
+        for (int i0 = tid; i0 < total; i0 += U * NT) {
+            uint4 v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const typename VA::At a = VA::at(ntiles, min(i0 + u * NT, total - 1));
+                if (row_exists(G, B, a.r))
+                    v[u] = *reinterpret_cast<const uint4*>(
+                        global_row(G, B, state, a.r) + (long long)(B.x0 / 32 + a.t) * VA::TE + a.q * VA::EV);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (i0 + u * NT >= total) break;
+                const typename VA::At a = VA::at(ntiles, i0 + u * NT);
+                if (!row_exists(G, B, a.r)) continue;
+                if (NARROW && a.p < 0) {
+                    const float* z = reinterpret_cast<const float*>(&v[u]);
+                    float* d = (a.p == -2 ? sps : sph) + a.r * RW + a.c + 1;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (a.c + e < w) d[e] = z[e];
+                } else {
+                    const S* q = reinterpret_cast<const S*>(&v[u]);
+                    float* d = pop + a.r * ROWF + a.p * RW + a.c + 1;
+#pragma unroll
+                    for (int e = 0; e < VA::EV; ++e)
+                        if (a.c + e < w) d[e] = narrow_to_f_or_self(q[e]);
+                }
+            }
+        }
+        constexpr int GP = PL + (NARROW ? 2 : 0);            // planes of a ghost column
+        for (int i = tid; i < (h + 2) * 2 * GP; i += NT) {
+            const int r = i / (2 * GP), side = i / GP % 2, p = i % GP;
+            const int c = side ? w : -1, gx = B.x0 + c;
+            if (!row_exists(G, B, r) || (G.wall_x && (gx < 0 || gx >= G.nx))) continue;
+            const int x = map_col(gx, G);
+            const S* tile = global_row(G, B, state, r) + (long long)(x >> 5) * VA::TE;
+            if (p >= PL)
+                gz[r * 4 + 2 * side + p - PL] =
+                    reinterpret_cast<const float*>(tile)[32 * (p - PL) + (x & 31)];
+            else
+                pop[r * ROWF + p * RW + c + 1] = narrow_to_f_or_self(
+                    tile[Tile<S>::P0 + (p + (SHEAR ? 9 : 0)) * 32 + (x & 31)]);
+        }
+    }
+}
+
+// Write a block's own nodes back (FP32 storage; the padding columns of a row's last tile stay as
+// they are).
+template <int V>
+__device__ __noinline__ void store_block(float* state, Geometry G, Block B, const float* pop)
+{
+    using VA = TileVec<float, V>;
+    constexpr int ROWF = row_floats<V>();
+    const int w = B.w, ntiles = (w + 31) / 32, total = B.h * ntiles * VA::TV;
+    for (int i = threadIdx.x; i < total; i += NT) {
+        typename VA::At a = VA::at(ntiles, i);
+        ++a.r;
+        float* to = global_row(G, B, state, a.r) + (long long)(B.x0 / 32 + a.t) * VA::TE + a.q * 4;
+        const float* q = pop + a.r * ROWF + a.p * RW + a.c + 1;
+        if (a.c + 4 <= w) *reinterpret_cast<float4*>(to) = make_float4(q[0], q[1], q[2], q[3]);
+        else
+            for (int e = 0; a.c + e < w; ++e) to[e] = q[e];
+    }
+}
+
+// A run of L.nsteps steps of this block.
 template <typename S, int V, class T>
-__global__ void __launch_bounds__(NT, 1)
-resident_kernel(S* __restrict__ state, Geometry G, Consts<float> K, ResidentLaunch L)
+__device__ __forceinline__ void resident_body(S* __restrict__ state, const Geometry& G,
+                                              const Consts<float>& K, const ResidentGrid& D,
+                                              const ResidentLaunch& L)
 {
     constexpr bool SRT = (V & kVarSRT) != 0;
     constexpr bool SHEAR = (V & kVarShear) != 0;
@@ -344,50 +508,35 @@ resident_kernel(S* __restrict__ state, Geometry G, Consts<float> K, ResidentLaun
     float* swirl = gz + (NARROW ? rows * 4 : 0);  // imposed flow: [rows][2] sin, cos of the rows
     const Lists tb = lists_at(swirl + (SHEAR ? rows * 2 : 0), L.hmax, L.tab);
     __shared__ int dead;
-    __shared__ int nbox[8];                       // first mailbox entry of the neighbours
+    __shared__ int nbox[16];                      // first mailbox entry of the neighbours
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const Block B = block_of(G, L);
+    const Block B = block_of(G, D);
     const int h = B.h, w = B.w;
     if (tid == 0) dead = 0;
-    if (tid < 8) {
-        const int d = tid < 4 ? tid : tid + 1;
-        const int s2 = (B.strip + d % 3 - 1 + L.nstrip) % L.nstrip;
-        const int g2 = (B.seg + d / 3 - 1 + L.nseg) % L.nseg;
-        nbox[tid] = (g2 * L.nstrip + s2) * L.box_entries;
+    if (tid < 15) {
+        const int dx = tid % 5 - 2, dy = tid / 5 - 1;
+        if (dx >= -reach<V>() && dx <= reach<V>() && (dx || dy)) {
+            const Neighbour N = neighbour(G, B, D, dx, dy);
+            nbox[neighbour_code<V>(dx, dy)] =
+                (D.block0 + N.seg * D.nstrip + N.strip) * L.box_entries;
+        }
     }
     const int words = (int)list_words(L.hmax, L.tab);
     const int* lists = L.lists + blockIdx.x * (2 + (size_t)words);
     const int nsend = lists[0], nrecv = lists[1], nring = ring_nodes(h);
+    if (nsend > L.tab || nrecv > L.tab) {   // never: list_capacity holds every list
+        if (tid == 0) atomicCAS(L.err, 0, 4);
+        return;
+    }
     for (int i = tid; i < words; i += NT) tb.node[i] = lists[2 + i];
 
-    // load the block and its ghost ring: 66 columns of every plane of every row
-    constexpr int TE = Tile<S>::ELEMS;
-    const long long row_elems = (long long)G.nstrips * TE;
-    for (int k = warp; k < (h + 2) * PL; k += NW) {
-        const int r = k / PL, p = k % PL;
-        const int gy = B.y0 + r - 1;
-        if (G.wall_y && (gy < 0 || gy >= G.ny)) continue;
-        const S* row = state + (long long)map_row(gy, G) * row_elems;
-        for (int c = lane - 1; c <= w; c += 32) {
-            const int gx = B.x0 + c;
-            if (G.wall_x && (gx < 0 || gx >= G.nx)) continue;
-            const int x = map_col(gx, G);
-            const S* q = row + (x >> 5) * TE + Tile<S>::P0 + (p + (SHEAR ? 9 : 0)) * 32 + (x & 31);
-            pop[r * ROWF + p * RW + c + 1] = narrow_to_f_or_self(*q);
-            if (NARROW && p < 2) {
-                const float* zp = reinterpret_cast<const float*>(row + (x >> 5) * TE);
-                const float z = zp[32 * p + (x & 31)];
-                if (c < 0 || c == w) gz[r * 4 + (c < 0 ? 0 : 2) + p] = z;
-                else (p ? sph : sps)[r * RW + c + 1] = z;
-            }
-        }
-    }
+    load_block<S, V>(state, G, B, pop, sps, sph, gz);
     if constexpr (SHEAR)
         for (int r = 1 + tid; r <= h; r += NT)
             sincospif(float(B.y0 + r - 1) * K.inv_ny - 0.5f, &swirl[2 * r], &swirl[2 * r + 1]);
     __syncthreads();
-    const bool xwall = G.wall_x && (B.strip == 0 || B.strip == L.nstrip - 1);
+    const bool xwall = G.wall_x && (B.strip == 0 || B.strip == D.nstrip - 1);
     const int cl = lane + (P == 1 ? 32 * (warp & 1) : 0);   // the lane's (first) column
     const bool actA = cl < w, actB = P == 2 && cl + 32 < w;
     const bool full = P == 2 ? w == 64 : w >= 32 * ((warp & 1) + 1);   // warp-uniform
@@ -405,9 +554,10 @@ resident_kernel(S* __restrict__ state, Geometry G, Consts<float> K, ResidentLaun
     // column whose moment stands beyond the strip's west / east end: a ghost, or at a wall the
     // end column itself
     const int cwest = G.wall_x && B.strip == 0 ? 0 : -1;
-    const int ceast = G.wall_x && B.strip == L.nstrip - 1 ? w - 1 : w;
+    const int ceast = G.wall_x && B.strip == D.nstrip - 1 ? w - 1 : w;
     constexpr int RPR = P == 2 ? NW : NW / 2;               // rows of a round
 
+    auto in_domain = [&](int r) { return row_exists(G, B, r); };
     // S for row r: phi and p* of its columns c0 .. c1 and, with `ends`, of the columns beyond its
     // ends (lane 0, 1 west p*, phi; lane 2, 3 east p*, phi)
     auto row_sums = [&](int r, int c0, int c1, bool ends) {
@@ -491,10 +641,6 @@ resident_kernel(S* __restrict__ state, Geometry G, Consts<float> K, ResidentLaun
         d[0] = sum;
         if (c == cwest) d[-1] = tree_sum(q, z);   // at a wall the end column itself
         if (c == ceast) d[1] = tree_sum(q, z);
-    };
-    auto in_domain = [&](int r) {
-        const int gy = B.y0 + r - 1;
-        return !(G.wall_y && (gy < 0 || gy >= G.ny));
     };
 
     for (int r = warp; r < h + 2; r += NW)
@@ -671,7 +817,7 @@ resident_kernel(S* __restrict__ state, Geometry G, Consts<float> K, ResidentLaun
                 const int i = min(i0 + k * NT, nsend - 1);
                 const float* o = pop + tb.soff[i];
                 const unsigned d = tb.sdst[i];
-                to[k] = nbox[d >> 13] + (int)(d & 8191u);
+                to[k] = nbox[d >> box_bits<V>()] + (int)(d & ((1u << box_bits<V>()) - 1));
                 a[k] = o[0];
                 b[k] = o[FO];
             }
@@ -762,23 +908,46 @@ resident_kernel(S* __restrict__ state, Geometry G, Consts<float> K, ResidentLaun
     }
 
     // write the block back; every neighbour has read its ghost ring (it has sent a message since)
-    for (int k = warp; k < h * PL; k += NW) {
-        const int r = 1 + k / PL, p = k % PL;
-        S* row = state + (long long)(B.y0 + r - 1) * row_elems;
-        for (int c = lane; c < w; c += 32) {
-            const int x = B.x0 + c;
-            S* tile = row + (x >> 5) * TE;
-            const float v = pop[r * ROWF + p * RW + c + 1];
-            if constexpr (NARROW) {
-                tile[Tile<S>::P0 + p * 32 + (x & 31)] = f_to_narrow<S>(v);
+    if constexpr (NARROW) {   // (in 16-byte accesses the whole time loop came out 14 % slower)
+        constexpr int TE = Tile<S>::ELEMS;
+        for (int k = warp; k < h * PL; k += NW) {
+            const int r = 1 + k / PL, p = k % PL;
+            for (int c = lane; c < w; c += 32) {
+                const int x = B.x0 + c;
+                S* tile = global_row(G, B, state, r) + (x >> 5) * TE;
+                tile[Tile<S>::P0 + p * 32 + (x & 31)] =
+                    f_to_narrow<S>(pop[r * ROWF + p * RW + c + 1]);
                 if (p < 2)   // the zeroth moments of the level before
                     reinterpret_cast<float*>(tile)[32 * p + (x & 31)] =
                         (p ? sph : sps)[r * RW + c + 1];
-            } else {
-                tile[Tile<S>::P0 + (p + (SHEAR ? 9 : 0)) * 32 + (x & 31)] = v;
             }
         }
+    } else {
+        store_block<V>(state, G, B, pop);
     }
+}
+
+template <typename S, int V, class T>
+__global__ void __launch_bounds__(NT, 1)
+resident_kernel(S* __restrict__ state, Geometry G, Consts<float> K, ResidentGrid D,
+                ResidentLaunch L)
+{
+    resident_body<S, V, T>(state, G, K, D, L);
+}
+
+// Many grids in one launch: block b runs its part of case case_of[b].
+template <typename S, int V>
+__global__ void __launch_bounds__(NT, 1)
+resident_batch_kernel(S* __restrict__ base, const ResidentCase* __restrict__ cases,
+                      const int* __restrict__ case_of, int parity, ResidentLaunch L)
+{
+    __shared__ Consts<float> K;
+    const ResidentCase& c = cases[case_of[blockIdx.x]];
+    for (int i = threadIdx.x; i < (int)(sizeof(K) / 4); i += NT)
+        reinterpret_cast<int*>(&K)[i] = reinterpret_cast<const int*>(&c.K)[i];
+    __syncthreads();
+    const Geometry G = c.G;
+    resident_body<S, V, F2>(base + c.off[parity], G, K, c.D, L);
 }
 
 template <typename S, int V>
@@ -801,68 +970,108 @@ const void* resident_fn(int hmax)
     return (const void*)resident_kernel<S, V, F2>;
 }
 
+// Entries of a block's send or receive list: nine populations of each node of the two outermost
+// rings with a source (or a taker) on the other side, three more a side row towards the block
+// beyond a single-column strip, and the corners.
+template <int V>
+constexpr int list_capacity(int hmax)
+{
+    return (9 * (2 * (64 + 2) + 2 * (hmax + 2)) + (reach<V>() == 2 ? 6 * (hmax + 2) : 0) + 128 +
+            3) & ~3;
+}
+constexpr int mailbox_entries(int hmax) { return 36 * RW + 36 * (hmax > 2 ? hmax - 2 : 0); }
+
+// Dynamic shared memory a block may have (the current device), and whether `fn` may be launched
+// with it.
+int most_smem()
+{
+    int dev = 0, most = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return most - 1024;   // the static part and the system's own
+}
+bool can_launch(const void* fn, size_t smem, int most)
+{
+    int nb = 0;
+    const bool ok =
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most) ==
+            cudaSuccess &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, NT, smem) == cudaSuccess && nb >= 1;
+    cudaGetLastError();
+    return ok;
+}
+
+// Blocks of at most `hmax` rows fit in shared memory and in the lists' 16-bit offsets.
+template <typename S, int V>
+bool rows_fit(int hmax, int most)
+{
+    return resident_smem<S, V>(hmax, list_capacity<V>(hmax)) <= (size_t)most &&
+           (hmax + 2) * row_floats<V>() <= 65535 &&
+           mailbox_entries(hmax) <= 1 << box_bits<V>();
+}
+
+// A grid's split needs two rows in every block, and strips whose reach the neighbour list covers.
+template <int V>
+bool grid_splits(const Geometry& G, int nstrip)
+{
+    const int last = G.nx - (nstrip - 1) * 64;
+    return G.ny >= 2 && (last >= 2 || (last == 1 && nstrip >= 2 && reach<V>() == 2));
+}
+
+template <typename S, int V>
+void fill_sizes(int nblocks, int hmax, ResidentSizes* z)
+{
+    z->nblocks = nblocks;
+    z->hmax = hmax;
+    z->tab = list_capacity<V>(hmax);
+    z->box_entries = mailbox_entries(hmax);
+    z->smem = resident_smem<S, V>(hmax, z->tab);
+    z->box_bytes = (size_t)2 * nblocks * z->box_entries * sizeof(ulonglong2);
+    z->list_bytes = (size_t)nblocks * (2 + list_words(hmax, z->tab)) * 4;
+}
+
+ResidentLaunch launch_args(const ResidentSizes& z, void* box, void* lists, int nsteps, int flow_sign,
+                           unsigned tag0, int* err)
+{
+    ResidentLaunch L = {};
+    L.hmax = z.hmax;
+    L.tab = z.tab;
+    L.box_entries = z.box_entries;
+    L.nsteps = nsteps;
+    L.flow_sign = flow_sign;
+    L.tag0 = tag0;
+    L.box = static_cast<ulonglong2*>(box);
+    L.lists = static_cast<int*>(lists);
+    L.err = err;
+    return L;
+}
+
 }  // namespace
 
 template <typename S, int V>
 bool resident_plan(const Geometry& G, int nsm, ResidentPlan* out)
 {
     const int nstrip = (G.nx + 63) / 64;
-    // a population crosses at most one block a step, and ghosts are sourced within the next
-    // block, where every block has at least two rows and columns
-    if (G.nx - (nstrip - 1) * 64 < 2 || G.ny < 2 || nstrip > nsm) return false;
+    if (!grid_splits<V>(G, nstrip) || nstrip > nsm) return false;
     const int nseg = nsm / nstrip < G.ny / 2 ? nsm / nstrip : G.ny / 2;
-    const int hmax = (G.ny + nseg - 1) / nseg;
-    const int tab = (9 * (2 * (64 + 2) + 2 * (hmax + 2)) + 128 + 3) & ~3;
-    const size_t smem = resident_smem<S, V>(hmax, tab);
-    // 16-bit offsets and 13-bit mailbox indices of the lists
-    if ((hmax + 2) * row_floats<V>() > 65535 || 36 * RW + 36 * hmax > 8191) return false;
-    int dev = 0, most = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
-        return false;
-    if (smem + 64 > (size_t)most) return false;
-    const void* fn = resident_fn<S, V>(hmax);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - 1024) !=
-        cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, NT, smem) != cudaSuccess || nb < 1) {
-        cudaGetLastError();
-        return false;
-    }
-    out->nstrip = nstrip;
-    out->nseg = nseg;
-    out->hmax = hmax;
-    out->tab = tab;
-    out->box_entries = 36 * RW + 36 * (hmax > 2 ? hmax - 2 : 0);
-    out->smem = smem;
-    out->box_bytes = (size_t)2 * nstrip * nseg * out->box_entries * sizeof(ulonglong2);
-    out->list_bytes = (size_t)nstrip * nseg * (2 + list_words(hmax, tab)) * 4;
-    return true;
-}
-
-static ResidentLaunch launch_args(const ResidentPlan& P, void* box, void* lists)
-{
-    ResidentLaunch L = {};
-    L.nstrip = P.nstrip;
-    L.nseg = P.nseg;
-    L.hmax = P.hmax;
-    L.tab = P.tab;
-    L.box_entries = P.box_entries;
-    L.box = static_cast<ulonglong2*>(box);
-    L.lists = static_cast<int*>(lists);
-    return L;
+    const int hmax = (G.ny + nseg - 1) / nseg, most = most_smem();
+    if (!rows_fit<S, V>(hmax, most)) return false;
+    out->D = {nstrip, nseg, 0};
+    fill_sizes<S, V>(nstrip * nseg, hmax, &out->Z);
+    return can_launch(resident_fn<S, V>(hmax), out->Z.smem, most);
 }
 
 template <typename S, int V>
 cudaError_t prepare_resident(const Geometry& G, const ResidentPlan& P, void* box, void* lists,
                              cudaStream_t st)
 {
-    cudaError_t e = cudaMemsetAsync(box, 0, P.box_bytes, st);
+    cudaError_t e = cudaMemsetAsync(box, 0, P.Z.box_bytes, st);
     if (e != cudaSuccess) return e;
-    resident_lists_kernel<V><<<P.nstrip * P.nseg, NT, 0, st>>>(G, launch_args(P, box, lists));
+    resident_lists_kernel<V><<<P.Z.nblocks, NT, 0, st>>>(
+        G, P.D, launch_args(P.Z, box, lists, 0, 1, 0, nullptr));
     return cudaGetLastError();
 }
 
@@ -871,17 +1080,98 @@ cudaError_t launch_resident(void* state, const Geometry& G, const Consts<float>&
                             const ResidentPlan& P, int nsteps, int flow_sign, unsigned tag0,
                             void* box, void* lists, int* err, cudaStream_t st)
 {
-    ResidentLaunch L = launch_args(P, box, lists);
-    L.nsteps = nsteps;
-    L.flow_sign = flow_sign;
-    L.tag0 = tag0;
-    L.err = err;
+    ResidentLaunch L = launch_args(P.Z, box, lists, nsteps, flow_sign, tag0, err);
     S* s = static_cast<S*>(state);
     Geometry g = G;
     Consts<float> k = K;
-    void* args[] = {(void*)&s, (void*)&g, (void*)&k, (void*)&L};
-    return cudaLaunchCooperativeKernel(resident_fn<S, V>(P.hmax), dim3(P.nstrip * P.nseg),
-                                       dim3(NT), args, P.smem, st);
+    ResidentGrid d = P.D;
+    void* args[] = {(void*)&s, (void*)&g, (void*)&k, (void*)&d, (void*)&L};
+    return cudaLaunchCooperativeKernel(resident_fn<S, V>(P.Z.hmax), dim3(P.Z.nblocks), dim3(NT),
+                                       args, P.Z.smem, st);
+}
+
+// Waves of a batch.  The taller its blocks, the less of a step a wave spends in the exchange, so
+// every case first gets the fewest blocks that its rows fit in; cases of like block heights share a
+// wave (its step takes as long as its tallest block), and the blocks a wave has left go to the
+// cases with its tallest.
+template <typename S, int V>
+bool resident_batch_plan(const Geometry* G, int ncases, int nsm, std::vector<ResidentWave>* waves)
+{
+    const int most = most_smem();
+    int cap = 0;
+    while (rows_fit<S, V>(cap + 1, most)) ++cap;
+    if (cap < 2) return false;
+    struct Part { int c, nstrip, nseg, h; };
+    std::vector<Part> parts;
+    for (int c = 0; c < ncases; ++c) {
+        Part p = {c, (G[c].nx + 63) / 64, (G[c].ny + cap - 1) / cap, 0};
+        p.h = (G[c].ny + p.nseg - 1) / p.nseg;
+        if (!grid_splits<V>(G[c], p.nstrip) || p.nstrip * p.nseg > nsm) return false;
+        parts.push_back(p);
+    }
+    std::stable_sort(parts.begin(), parts.end(),
+                     [](const Part& a, const Part& b) { return a.h > b.h; });
+    std::vector<std::vector<Part>> bins;
+    std::vector<int> used;
+    for (const Part& p : parts) {
+        size_t w = 0;
+        while (w < bins.size() && used[w] + p.nstrip * p.nseg > nsm) ++w;
+        if (w == bins.size()) {
+            bins.push_back({});
+            used.push_back(0);
+        }
+        bins[w].push_back(p);
+        used[w] += p.nstrip * p.nseg;
+    }
+    for (size_t w = 0; w < bins.size(); ++w) {
+        std::vector<Part>& b = bins[w];
+        for (;;) {
+            Part* t = &b[0];
+            for (Part& p : b)
+                if (p.h > t->h) t = &p;
+            // one segment more at a time shortens the tallest only now and then: go to the next
+            // count that does
+            int n = t->nseg + 1;
+            while (n <= G[t->c].ny / 2 && (G[t->c].ny + n - 1) / n == t->h) ++n;
+            if (n > G[t->c].ny / 2 || used[w] + (n - t->nseg) * t->nstrip > nsm) break;
+            used[w] += (n - t->nseg) * t->nstrip;
+            t->nseg = n;
+            t->h = (G[t->c].ny + n - 1) / n;
+        }
+        ResidentWave W;
+        int nblocks = 0, hmax = 2;
+        for (const Part& p : b) {
+            W.cases.push_back(p.c);
+            W.D.push_back({p.nstrip, p.nseg, nblocks});
+            nblocks += p.nstrip * p.nseg;
+            hmax = std::max(hmax, p.h);
+        }
+        fill_sizes<S, V>(nblocks, hmax, &W.Z);
+        if (!can_launch((const void*)resident_batch_kernel<S, V>, W.Z.smem, most)) return false;
+        waves->push_back(W);
+    }
+    return true;
+}
+
+template <typename S, int V>
+cudaError_t prepare_resident_batch(const ResidentSizes& Z, const ResidentCase* cases,
+                                   const int* case_of, void* lists, cudaStream_t st)
+{
+    resident_batch_lists_kernel<V><<<Z.nblocks, NT, 0, st>>>(
+        cases, case_of, launch_args(Z, nullptr, lists, 0, 1, 0, nullptr));
+    return cudaGetLastError();
+}
+
+template <typename S, int V>
+cudaError_t launch_resident_batch(void* base, const ResidentSizes& Z, const ResidentCase* cases,
+                                  const int* case_of, int parity, int nsteps, unsigned tag0,
+                                  void* box, void* lists, int* err, cudaStream_t st)
+{
+    ResidentLaunch L = launch_args(Z, box, lists, nsteps, 1, tag0, err);
+    S* s = static_cast<S*>(base);
+    void* args[] = {(void*)&s, (void*)&cases, (void*)&case_of, (void*)&parity, (void*)&L};
+    return cudaLaunchCooperativeKernel((const void*)resident_batch_kernel<S, V>, dim3(Z.nblocks),
+                                       dim3(NT), args, Z.smem, st);
 }
 
 #define CMLBM_INSTANTIATE_RESIDENT(S, V)                                                          \
@@ -891,6 +1181,16 @@ cudaError_t launch_resident(void* state, const Geometry& G, const Consts<float>&
     template cudaError_t launch_resident<S, V>(void*, const Geometry&, const Consts<float>&,    \
                                                const ResidentPlan&, int, int, unsigned, void*,  \
                                                void*, int*, cudaStream_t);
+#define CMLBM_INSTANTIATE_RESIDENT_BATCH(S, V)                                                    \
+    template bool resident_batch_plan<S, V>(const Geometry*, int, int,                          \
+                                            std::vector<ResidentWave>*);                        \
+    template cudaError_t prepare_resident_batch<S, V>(const ResidentSizes&,                     \
+                                                      const ResidentCase*, const int*, void*,   \
+                                                      cudaStream_t);                            \
+    template cudaError_t launch_resident_batch<S, V>(void*, const ResidentSizes&,               \
+                                                     const ResidentCase*, const int*, int, int, \
+                                                     unsigned, void*, void*, int*,              \
+                                                     cudaStream_t);
 CMLBM_INSTANTIATE_RESIDENT(float, 0)
 CMLBM_INSTANTIATE_RESIDENT(float, 1)
 CMLBM_INSTANTIATE_RESIDENT(float, 2)
@@ -899,6 +1199,13 @@ CMLBM_INSTANTIATE_RESIDENT(float, 4)
 CMLBM_INSTANTIATE_RESIDENT(float, 5)
 CMLBM_INSTANTIATE_RESIDENT(__half, 0)
 CMLBM_INSTANTIATE_RESIDENT(__nv_bfloat16, 0)
+CMLBM_INSTANTIATE_RESIDENT_BATCH(float, 0)
+CMLBM_INSTANTIATE_RESIDENT_BATCH(float, 1)
+CMLBM_INSTANTIATE_RESIDENT_BATCH(float, 4)
+CMLBM_INSTANTIATE_RESIDENT_BATCH(float, 5)
+CMLBM_INSTANTIATE_RESIDENT_BATCH(__half, 0)
+CMLBM_INSTANTIATE_RESIDENT_BATCH(__nv_bfloat16, 0)
 #undef CMLBM_INSTANTIATE_RESIDENT
+#undef CMLBM_INSTANTIATE_RESIDENT_BATCH
 
 }  // namespace cmlbm

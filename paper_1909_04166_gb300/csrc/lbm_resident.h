@@ -1,7 +1,9 @@
-// The resident step kernel (lbm_resident.cu): its plan for a grid and its launch.
+// The resident step kernel (lbm_resident.cu): its plans for a grid or a batch, and its launches.
 #pragma once
 
 #include <cuda_runtime.h>
+
+#include <vector>
 
 #include "lbm_device.cuh"
 
@@ -9,10 +11,14 @@ namespace cmlbm {
 
 constexpr int kResidentWarps = 16;   // warps of a block; one block per SM
 
-// Split of a grid into blocks of one strip of 64 columns and at most hmax rows.
-struct ResidentPlan {
-    int nstrip, nseg;     // blocks = nstrip * nseg
-    int hmax;             // rows of the tallest block
+// A grid's blocks: nstrip strips of 64 columns times nseg row segments, numbered from block0.
+struct ResidentGrid {
+    int nstrip, nseg, block0;
+};
+
+// What a launch of blocks of at most hmax rows takes.
+struct ResidentSizes {
+    int nblocks, hmax;
     int tab;              // capacity of a block's send and receive lists
     int box_entries;      // 16-byte words of a block's mailbox (one of two)
     size_t smem;          // dynamic shared memory of a block
@@ -20,8 +26,28 @@ struct ResidentPlan {
     size_t list_bytes;    // the exchange lists of all blocks
 };
 
+struct ResidentPlan {
+    ResidentGrid D;
+    ResidentSizes Z;
+};
+
+// One case of a batch as the kernel sees it (off: element offsets of its two buffers).
+struct ResidentCase {
+    Geometry G;
+    ResidentGrid D;
+    long long off[2];
+    Consts<float> K;
+};
+
+// Cases of a batch whose blocks fit on the device at once: indices and splits, in block order.
+struct ResidentWave {
+    std::vector<int> cases;
+    std::vector<ResidentGrid> D;
+    ResidentSizes Z;
+};
+
 struct ResidentLaunch {
-    int nstrip, nseg, hmax, tab, box_entries;
+    int hmax, tab, box_entries;
     int nsteps;
     int flow_sign;        // imposed flow: +1, or -1 once reversed
     unsigned tag0;        // messages of step s carry tag0 + 1 + s
@@ -31,7 +57,7 @@ struct ResidentLaunch {
 };
 
 // Plan for a grid on a device of nsm SMs (the current device); false where its state does not
-// fit in their shared memory or a block would be one node wide.
+// fit in their shared memory, a block would have a single row, or the grid a single column.
 template <typename S, int V>
 bool resident_plan(const Geometry&, int nsm, ResidentPlan*);
 
@@ -46,5 +72,18 @@ template <typename S, int V>
 cudaError_t launch_resident(void* state, const Geometry&, const Consts<float>&,
                             const ResidentPlan&, int nsteps, int flow_sign, unsigned tag0,
                             void* box, void* lists, int* err, cudaStream_t);
+
+// The same for a batch, one launch per wave; false where a case does not fit.  The waves of a
+// batch may share one set of mailboxes (zeroed by the caller), with tags that continue from launch
+// to launch; case_of[b] is the index into `cases` of block b of the wave.
+template <typename S, int V>
+bool resident_batch_plan(const Geometry*, int ncases, int nsm, std::vector<ResidentWave>*);
+template <typename S, int V>
+cudaError_t prepare_resident_batch(const ResidentSizes&, const ResidentCase* cases,
+                                   const int* case_of, void* lists, cudaStream_t);
+template <typename S, int V>
+cudaError_t launch_resident_batch(void* base, const ResidentSizes&, const ResidentCase* cases,
+                                  const int* case_of, int parity, int nsteps, unsigned tag0,
+                                  void* box, void* lists, int* err, cudaStream_t);
 
 }  // namespace cmlbm

@@ -2,7 +2,7 @@
 against one launch per step: the same state, bit for bit.
 
 Blocks of 64 columns exchange their borders through mailboxes and fold rows that several rounds of
-warps share, so the shapes are those where this can go wrong: strips of 2, 63 and 64 columns, blocks
+warps share, so the shapes are those where this can go wrong: strips of 1, 2, 63 and 64 columns, blocks
 of 2 rows, of half a row per warp (at most 8 rows) and of one, two and several rounds, one block
 that is its own neighbour, every side kind and its corners.  A run in place leaves the state in the
 buffer it was in; an odd run of the other forms moves it to the other one.
@@ -28,6 +28,9 @@ SHAPES = [
     (128, 700, (1, 2), (2, 1)),
     (161, 481, (2, 2), (1, 1)),
     (257 + 63, 640, (0, 0), (0, 0)),
+    (65, 40, (0, 0), (0, 0)),           # a last strip of one column
+    (129, 200, (0, 0), (2, 1)),
+    (65, 33, (1, 2), (0, 0)),
     (256, 1024, (0, 0), (1, 1)),
 ]
 
@@ -81,8 +84,47 @@ def test_resident_imposed_flow_across_the_reversal(L0):
     assert np.array_equal(out[0], out[1])
 
 
-def test_grids_beyond_shared_memory_and_one_node_strips_take_the_other_forms():
-    for nx, ny in ((65, 40), (1, 30), (30, 1), (700, 900)):
+@pytest.mark.parametrize("layout", [lbm.LBM_BATCH_AS_GIVEN, lbm.LBM_BATCH_FEWEST_COLUMNS])
+@pytest.mark.parametrize("precision", ["fp32", "fp16", "bf16"])
+def test_resident_batches_match_graph_replays(precision, layout):
+    """Cases of several waves, among them single-column strips and a case of one block."""
+    cases = W.ensemble(40) + [
+        W.random_drop(nx, ny, seed=nx, wall_x=bx, wall_y=by, rho_ratio=50.0, gravity=1e-6)
+        for nx, ny, bx, by in ((65, 70, 0, 0), (193, 65, 0, 2), (129, 65, 2, 1), (2, 2, 0, 0),
+                               (64, 300, 1, 0), (33, 20, 0, 1))]
+    outs = []
+    for resident in (True, False):
+        with lbm.Batch(cases, precision=precision, layout=layout) as b:
+            b.init_all()
+            if not resident:
+                lbm.lbm_batch_set_persistent(b.b, 0)
+            for n in (65, 1, 2, 80):
+                b.step(n)
+            lbm.lbm_batch_check(b.b)
+            outs.append([b.populations(i) for i in range(len(cases))])
+    for (ga, fa), (gb, fb) in zip(*outs):
+        assert np.array_equal(ga, gb) and np.array_equal(fa, fb)
+
+
+@pytest.mark.parametrize("collision,sigma_model", [(1, 0), (0, 1), (1, 1)])
+def test_resident_batch_variants(collision, sigma_model):
+    cases = [W.random_drop(nx, ny, seed=nx, wall_y=1, rho_ratio=10.0, gravity=1e-6,
+                           collision=collision, sigma_model=sigma_model, beta=0.4, psi0=0.2,
+                           gradpsi_x=1e-3) for nx, ny in ((75, 66), (130, 200), (65, 40))]
+    outs = []
+    for resident in (True, False):
+        with lbm.Batch(cases, precision="fp32") as b:
+            b.init_all()
+            if not resident:
+                lbm.lbm_batch_set_persistent(b.b, 0)
+            b.step(33).step(40)
+            outs.append([b.populations(i) for i in range(len(cases))])
+    for (ga, fa), (gb, fb) in zip(*outs):
+        assert np.array_equal(ga, gb) and np.array_equal(fa, fb)
+
+
+def test_grids_beyond_shared_memory_and_of_one_node_take_the_other_forms():
+    for nx, ny in ((1, 30), (30, 1), (700, 900)):
         case = W.random_drop(nx, ny, seed=4, wall_y=1, rho_ratio=10.0)
         with lbm.Simulation(case, precision="fp32") as sim:
             sim.init_case()

@@ -378,7 +378,7 @@ int lbm_diagnostics_noalloc(const double* phi, const double* p, const double* ux
  * stored transposed is stepped as its problem reflected across the diagonal (grid, boundary
  * kinds, gradients and body force with x and y exchanged), whose solution the D2Q9 scheme of
  * Secs. 3 and 5 maps onto the reflected one.  All fields and populations are passed in the
- * case's own orientation; the transposes run on the host in those calls.  A case stored as
+ * case's own orientation; the transposes run in those calls.  A case stored as
  * given evolves bitwise as in its own context; a transposed one agrees with it up to the
  * rounding of the reflected evaluation order.
  * ------------------------------------------------------------------------------------------- */

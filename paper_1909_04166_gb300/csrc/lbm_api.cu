@@ -439,7 +439,7 @@ int run_fields(lbm_ctx* c, double* phi, double* p, double* ux, double* uy, doubl
         using R = decltype(r);
         return launch_fields<R, decltype(s)>(cur_state(c), c->G, kref<R>(c),
                                              flow_sign_at(c, c->steps), phi, p, ux, uy, rho,
-                                             c->st);
+                                             0, c->st);
     });
     return e == cudaSuccess ? LBM_OK : cuda_fail(c, e);
 }

@@ -9,7 +9,8 @@
 // (x <-> y for the grid, the boundary kinds, the temperature and surfactant gradients and the
 // body force; populations 1 <-> 2, 3 <-> 4, 6 <-> 8), which the D2Q9 scheme of Secs. 3 and 5
 // maps onto the reflected solution.  Fields and populations cross the boundary in the case's
-// own orientation; the transposes run on the host.
+// own orientation; the transposes run on the host, but for the fields read out, which the device
+// writes in that orientation.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -598,28 +599,21 @@ int lbm_batch_get_fields(lbm_batch* b, int32_t c, double* phi, double* p, double
     cudaSetDevice(b->device);
     const HostCase& hc = b->cases[c];
     const size_t N = (size_t)hc.nodes, B = N * sizeof(double);
-    double* d = b->scratch;
+    // device arrays of the fields asked for, in the case's own orientation: a transposed case's
+    // stored u_x is its own u_y
+    double* h[5] = {phi, p, ux, uy, rho};
+    double* d[5];
+    for (int k = 0; k < 5; ++k) d[k] = h[k] ? b->scratch + k * N : nullptr;
     cudaError_t e = with_types(b->precision, [&](auto r, auto s) {
         using R = decltype(r);
-        return launch_fields<R, decltype(s)>(case_state(b, c), hc.G, kref<R>(hc), 0, d, d + N,
-                                             d + 2 * N, d + 3 * N, d + 4 * N, b->st);
+        return launch_fields<R, decltype(s)>(case_state(b, c), hc.G, kref<R>(hc), 0, d[0], d[1],
+                                             hc.tr ? d[3] : d[2], hc.tr ? d[2] : d[3], d[4],
+                                             hc.tr ? 1 : 0, b->st);
     });
-    // destination of stored field k (phi, p, u_x, u_y, rho of the stored grid): a transposed
-    // case's stored u_x is its own u_y
-    double* own[5] = {phi, p, hc.tr ? uy : ux, hc.tr ? ux : uy, rho};
-    double* h[5] = {own[0], own[1], own[2], own[3], own[4]};
-    std::vector<double> t;
-    if (hc.tr) {   // fetch the stored fields, then transpose each into the case's orientation
-        t.resize(5 * N);
-        for (int k = 0; k < 5; ++k) h[k] = own[k] ? t.data() + k * N : nullptr;
-    }
     for (int k = 0; k < 5 && e == cudaSuccess; ++k)
-        if (h[k]) e = cudaMemcpyAsync(h[k], d + k * N, B, cudaMemcpyDeviceToHost, b->st);
+        if (h[k]) e = cudaMemcpyAsync(h[k], d[k], B, cudaMemcpyDeviceToHost, b->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
     if (e != cudaSuccess) return fail_cuda(b, e);
-    if (hc.tr)
-        for (int k = 0; k < 5; ++k)
-            if (own[k]) transpose(t.data() + k * N, hc.P.nx, hc.P.ny, own[k]);
     return check_err(b);
 }
 

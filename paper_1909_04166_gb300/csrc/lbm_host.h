@@ -50,7 +50,7 @@ cudaError_t launch_init(const double*, const double*, const double*, const doubl
                         const Geometry&, const Consts<R>&, cudaStream_t);
 template <typename R, typename S>
 cudaError_t launch_fields(const void*, const Geometry&, const Consts<R>&, int, double*, double*,
-                          double*, double*, double*, cudaStream_t);
+                          double*, double*, double*, int transposed, cudaStream_t);
 template <typename R, typename S>
 cudaError_t launch_pack(const void*, double*, const Geometry&, const Consts<R>&, cudaStream_t);
 template <typename R, typename S>

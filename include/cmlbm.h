@@ -236,7 +236,8 @@ int lbm_set_graphs(lbm_ctx* ctx, int32_t enable);
 
 /* The multi-step kernel of lbm_step: enable = 1 uses it wherever the grid's warps fit on the
  * device at once, 0 never, 2 (automatic) where they fit and the warp segments are at least 3
- * rows tall (shorter segments spend more of a step in the waits between steps).  Results are
+ * rows tall, 12 for the interface lattice alone (shorter segments spend more of a step in the
+ * waits between steps).  Results are
  * identical.  Default: 2 with LBM_FP32 storage, 0 with the others (where it measured slower
  * than graph replays).  A call with 0 or 1 also keeps runs from the resident kernel (lbm_step),
  * a call with 2 allows it again.  Other values: LBM_ERR_ARG. */

@@ -71,6 +71,10 @@ constexpr int kMaxWarpsPerSm = 64;
 // 512 x 256, 2 rows, 8.9 against 7.1; Laplace 64 x 64, 1 row, 5.9 against 3.7).
 constexpr int kMultiAuto = 2;
 constexpr int kMultiAutoMinRows = 3;
+// The interface lattice alone moves half as much a row, so that the waits weigh more: 830 x 830
+// (6 rows) 13.3 against 12.1 us a step, 1024 x 1024 (9 rows) 17.1 against 16.1, 1300 x 1300 (16
+// rows) 26.2 against 26.5, 1600 x 1600 (23 rows) 35.7 against 36.5.
+constexpr int kMultiAutoMinRowsFlow = 12;
 
 template <typename R> const Consts<R>& kref(const lbm_ctx* c);
 template <> const Consts<double>& kref<double>(const lbm_ctx* c) { return c->Kd; }
@@ -179,7 +183,9 @@ bool multi_fits(const lbm_ctx* c)
 {
     if (!c->use_multi || c->multi_bps <= 0 || c->checked || c->cut_first_wait == 1) return false;
     // automatic: only with segments tall enough that a step outlasts the waits between steps
-    if (c->use_multi == kMultiAuto && c->seg_h < kMultiAutoMinRows) return false;
+    const int min_rows =
+        c->P.flow == LBM_FLOW_SHEAR ? kMultiAutoMinRowsFlow : kMultiAutoMinRows;
+    if (c->use_multi == kMultiAuto && c->seg_h < min_rows) return false;
     const int strips = with_variant(c->P.precision, c->variant, [&](auto r, auto s, auto v) {
         return step_warp_strips<decltype(r), decltype(s), decltype(v)::value>(c->G.nstrips);
     });

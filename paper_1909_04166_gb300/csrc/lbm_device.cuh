@@ -220,26 +220,39 @@ template <> __device__ __forceinline__ void sincospi_<float>(float v, float* s, 
 {
     sincospif(v, s, c);
 }
-template <typename R> __device__ __forceinline__ R rcp_(R v) { return R(1) / v; }
-template <> __device__ __forceinline__ float rcp_<float>(float v) { return __fdividef(1.0f, v); }
-__device__ __forceinline__ F2 rcp_(F2 v)
+// Reciprocal and reciprocal root of normal numbers, one instruction each: __fdividef(1, v) and
+// rsqrtf(v) also scale denormal arguments, which the update never passes, and give the same bits for
+// every normal v (compared over all of them).  One GB300, us a step: Rayleigh-Taylor 256 x 1024
+// 6.1 -> 5.9, impact 1501 x 501 19.8 -> 19.0, impact 2048 x 1024 with FP16 storage 55.3 -> 53.9.
+__device__ __forceinline__ float rcp_ftz(float v)
 {
-    return F2(__fdividef(1.0f, v.v.x), __fdividef(1.0f, v.v.y));
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
 }
-__device__ __forceinline__ F1 rcp_(F1 v) { return F1(__fdividef(1.0f, v.v)); }
+__device__ __forceinline__ float rsqrt_ftz(float v)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+template <typename R> __device__ __forceinline__ R rcp_(R v) { return R(1) / v; }
+template <> __device__ __forceinline__ float rcp_<float>(float v) { return rcp_ftz(v); }
+__device__ __forceinline__ F2 rcp_(F2 v) { return F2(rcp_ftz(v.v.x), rcp_ftz(v.v.y)); }
+__device__ __forceinline__ F1 rcp_(F1 v) { return F1(rcp_ftz(v.v)); }
 // sqrt(v) for v >= 0: exact in double; v * rsqrt(v) in float (0 for v = 0)
 template <typename R> __device__ __forceinline__ R norm_(R v) { return sqrt(v); }
 template <> __device__ __forceinline__ float norm_<float>(float v)
 {
-    return v * rsqrtf(fmaxf(v, 1e-37f));
+    return v * rsqrt_ftz(fmaxf(v, 1e-37f));
 }
 __device__ __forceinline__ F2 norm_(F2 v)
 {
-    return v * F2(rsqrtf(fmaxf(v.v.x, 1e-37f)), rsqrtf(fmaxf(v.v.y, 1e-37f)));
+    return v * F2(rsqrt_ftz(fmaxf(v.v.x, 1e-37f)), rsqrt_ftz(fmaxf(v.v.y, 1e-37f)));
 }
 __device__ __forceinline__ F1 norm_(F1 v)
 {
-    return v * F1(rsqrtf(fmaxf(v.v, 1e-37f)));
+    return v * F1(rsqrt_ftz(fmaxf(v.v, 1e-37f)));
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -26,8 +26,21 @@ static constexpr unsigned FULL = 0xffffffffu;
 enum : int { kVarSRT = 1, kVarShear = 2, kVarLangmuir = 4 };
 
 // Per-case constants in the compute precision R.  Derived on the host from lbm_params.
+// Constants of the double-precision update (node_macro_dp) with its fixed factors folded in: it
+// works with 12 grad phi and 12 H (the differences without their divisors), F_t / 6 and F_p / 3.
+struct Folded {
+    double mu3_b, dmu3;       // 3 mu = mu3_b + phi dmu3
+    double kt0, dktx, dkty;   // kappa-tilde / 864, of 12 * 12 from the differences and 6 from F_t / 6
+    double sharp;             // omega^phi M_phi 4 / W
+    double gx, gy;            // g / 6
+    double cs2_drho;          // c_s^2 (rho_A - rho_B) / 36
+    int forces;               // gravity, or a kappa-tilde that varies over the grid
+};
+template <typename R> struct FoldedOf {};
+template <> struct FoldedOf<double> { Folded F; };
+
 template <typename R>
-struct Consts {
+struct Consts : FoldedOf<R> {
     R rho_b, drho;       // rho = rho_b + phi drho                      (Sec. 2, linear interpolation)
     R mu_b, dmu;         // mu  = mu_b  + phi dmu
     R kt0, dktx, dkty;   // kappa-tilde(x, y) = kt0 + dktx x + dkty y   (kappa-tilde = 3/2 sigma W)
@@ -317,6 +330,15 @@ struct Macro {
     T Ftx, Fty, Fpx, Fpy;  // total force and net gradient pressure force
     T jx, jy;              // M_phi theta n, the interface first-order equilibrium moment
 };
+// In double precision also what its few-operations form hands on; jx, jy are then times omega^phi.
+template <>
+struct Macro<double> {
+    double rho, omega, ux, uy, p, Ftx, Fty, Fpx, Fpy, jx, jy;
+    double mx, my;         // rho c_s^2 u
+    double Ft6x, Ft6y;     // total force / 6
+    double Fp3x, Fp3y;     // net gradient pressure force / 3
+    double H;              // F_p . u / 3
+};
 
 // Forces and corrected fields of one node, from the phi and p* windows and the streamed g-bar
 // first moments (Sec. 2 properties and surface tension, Sec. 6.7 Marangoni components, Sec. 3
@@ -601,8 +623,9 @@ __device__ __forceinline__ void collide_ace_srt(T f[9], T phi, const Macro<T>& m
                                           fmad(ux2 * uy2, phi, c22)));
     // relaxation at one rate
     const T keep = T(R(1)) - om;
-    const T a = fmad(keep, c10, om * m.jx);
-    const T b = fmad(keep, c01, om * m.jy);
+    const T omj = std::is_same<T, double>::value ? T(R(1)) : om;   // (m.jx holds omega then)
+    const T a = fmad(keep, c10, omj * m.jx);
+    const T b = fmad(keep, c01, omj * m.jy);
     const T d20 = fmad(keep, c20, om * (third * phi));
     const T d02 = fmad(keep, c02, om * (third * phi));
     const T d11 = keep * c11, d21 = keep * c21, d12 = keep * c12;
@@ -654,6 +677,244 @@ __device__ __forceinline__ void collide_ace(T f[9], T phi, const Macro<T>& m, T 
     const T r22 = fmad(ninth, phi, fmad(ux2 + uy2, cp, fmad(two * uxy, fmad(uy, a, ux * b),
                                                              (ux2 * uy2) * phi)));
     raw_to_pop_fast(phi, r10, r01, r20, r02, r11, r21, r12, r22, f);
+}
+
+// ---------------------------------------------------------------------------------------------
+// The update in double precision.  Its unit takes an SM 19 cycles a warp instruction (64 at least
+// for a lone warp), so a step costs its number of operations and little else.  The formulas above
+// take about 310 a node; written as here they take about 210: differences without their divisors
+// and constants with the fixed factors folded in (Folded), the Laplacian as the Hessian's trace,
+// rho c^2 u from the corrected first moments, equilibria as products of one-dimensional moments.
+// One GB300, us a step: 64 x 64 16.2 -> 13.6, 45 x 77 16.2 -> 13.7, 200 x 100 23.0 -> 18.5, Marangoni
+// 300 x 200 50.6 -> 41.4; the error against a double-precision restatement stays its own rounding
+// level.  The FP32 forms keep their grouping: a long run amplifies any other roundings there.
+// ---------------------------------------------------------------------------------------------
+// 12 grad a.
+__device__ __forceinline__ void grad12(const Win<double>& a, double& gx, double& gy)
+{
+    const double d1 = a.ne - a.sw, d2 = a.se - a.nw;
+    gx = fmad(4.0, a.e - a.w, d1 + d2);
+    gy = fmad(4.0, a.n - a.s, d1 - d2);
+}
+// -12 grad a
+__device__ __forceinline__ void minus_grad12(const Win<double>& a, double& gx, double& gy)
+{
+    const double d1 = a.sw - a.ne, d2 = a.nw - a.se;
+    gx = fmad(4.0, a.w - a.e, d1 + d2);
+    gy = fmad(4.0, a.s - a.n, d1 - d2);
+}
+
+// The Hessian of one window, the 1-10-1 weighted second difference across the three rows
+// (columns): 12 h_xx, 12 h_yy and 4 h_xy.  Its trace is the isotropic Laplacian.  The second differences are sums of first differences, which are exact where a varies little.
+__device__ __forceinline__ void hessian12(const Win<double>& a, double& hxx, double& hyy,
+                                          double& hxy)
+{
+    const double ex = (a.e - a.c) + (a.w - a.c), ey = (a.n - a.c) + (a.s - a.c);
+    const double p1 = a.ne + a.sw, p2 = a.nw + a.se;
+    const double corners = fmad(-4.0, a.c, p1 + p2);
+    hxy = p1 - p2;
+    hxx = fmad(10.0, ex, fmad(-2.0, ey, corners));
+    hyy = fmad(10.0, ey, fmad(-2.0, ex, corners));
+}
+
+// First raw moments of nine populations.
+__device__ __forceinline__ void first_moments(const double q[9], double& mx, double& my)
+{
+    const double d1 = q[5] - q[7], d2 = q[6] - q[8];
+    mx = (q[1] - q[3]) + (d1 - d2);
+    my = (q[2] - q[4]) + (d1 + d2);
+}
+
+// Forces and corrected fields of one node (node_macro).
+template <bool LANGMUIR>
+__device__ __forceinline__ void node_macro_dp(const Win<double>& ph, const Win<double>& ps,
+                                              double jgx, double jgy, double xf, double yf,
+                                              const Consts<double>& K, Macro<double>& m)
+{
+    const double one = 1.0;
+    const double phi = ph.c;
+    m.rho = fmad(phi, K.drho, K.rho_b);
+    const double inv_rho = rcp_(m.rho);
+    // omega = 1 / (nu / c_s^2 + 1/2), nu = mu / rho
+    m.omega = rcp_(fmad(fmad(phi, K.F.dmu3, K.F.mu3_b), inv_rho, 0.5));
+
+    double gx, gy, hxx, hyy, hxy, mpx, mpy;
+    grad12(ph, gx, gy);
+    hessian12(ph, hxx, hyy, hxy);
+    minus_grad12(ps, mpx, mpy);
+
+    // regularised normal n = grad phi / (|grad phi| + 1e-6): defined everywhere, and rounding
+    // noise in the bulk phases cannot set its direction
+    const double g2 = fmad(gx, gx, gy * gy);
+    const double gm = sqrt(g2);
+    const double ig = rcp_(gm + 12e-6);
+    const double nx = gx * ig, ny = gy * ig;
+    // n.H.n - lap = (nx^2 - 1) h_xx + 2 nx ny h_xy + (ny^2 - 1) h_yy, times 12
+    const double ax = fmad(nx, nx, -1.0), ay = fmad(ny, ny, -1.0);
+    const double curv = fmad(ax, hxx, fmad(ay, hyy, (nx * ny) * (6.0 * hxy)));
+    const double bend = gm * curv;
+    // rho c_s^2 u = sum g-bar e + c_s^2 F_t / 2
+    if (!LANGMUIR && !K.F.forces) {
+        const double cap = K.F.kt0 * bend;              // -kappa-tilde |grad phi|^2 div n
+        m.Ft6x = cap * nx;
+        m.Ft6y = cap * ny;
+        m.mx = fmad(cap, nx, jgx);
+        m.my = fmad(cap, ny, jgy);
+    } else {
+        double kt, dktx, dkty;   // kappa-tilde and its gradient at the node
+        if constexpr (LANGMUIR) {
+            const double om = one - fmad(K.gpsx, xf, fmad(K.gpsy, yf, K.psi0));   // 1 - psi
+            kt = K.F.kt0 * fmad(K.beta, log_(om), one);
+            const double s = -K.F.kt0 * K.beta * rcp_(om);                           // d kt / d psi
+            dktx = s * K.gpsx;
+            dkty = s * K.gpsy;
+        } else {
+            kt = fmad(K.F.dktx, xf, fmad(K.F.dkty, yf, K.F.kt0));
+            dktx = K.F.dktx;
+            dkty = K.F.dkty;
+        }
+        const double cap = kt * bend;
+        const double mnd = -fmad(nx, dktx, ny * dkty);   // -n . grad kappa-tilde
+        const double dr = m.rho - K.rho_ref;
+        // + |grad phi|^2 (I - n n) grad kappa-tilde + gravity
+        m.Ft6x = fmad(cap, nx, fmad(g2, fmad(nx, mnd, dktx), dr * K.F.gx));
+        m.Ft6y = fmad(cap, ny, fmad(g2, fmad(ny, mnd, dkty), dr * K.F.gy));
+        m.mx = jgx + m.Ft6x;
+        m.my = jgy + m.Ft6y;
+    }
+    m.Fp3x = fmad(K.F.cs2_drho, gx, 1.0 / 36.0 * mpx);
+    m.Fp3y = fmad(K.F.cs2_drho, gy, 1.0 / 36.0 * mpy);
+    const double three_inv_rho = 3.0 * inv_rho;
+    m.ux = three_inv_rho * m.mx;
+    m.uy = three_inv_rho * m.my;
+    m.H = fmad(m.Fp3x, m.ux, m.Fp3y * m.uy);
+    m.p = fmad(1.5, m.H, ps.c);
+    const double theta_m = K.F.sharp * (phi * (one - phi));
+    m.jx = theta_m * nx;
+    m.jy = theta_m * ny;
+    // (for the single-relaxation form and the diagnostics)
+    m.Ftx = 6.0 * m.Ft6x;
+    m.Fty = 6.0 * m.Ft6y;
+    m.Fpx = 3.0 * m.Fp3x;
+    m.Fpy = 3.0 * m.Fp3y;
+}
+
+template <>
+__device__ __forceinline__ void node_macro<double, false>(
+    const Win<double>& ph, const Win<double>& ps, double jgx, double jgy, double xf, double yf,
+    const Consts<double>& K, Macro<double>& m)
+{
+    node_macro_dp<false>(ph, ps, jgx, jgy, xf, yf, K, m);
+}
+template <>
+__device__ __forceinline__ void node_macro<double, true>(
+    const Win<double>& ph, const Win<double>& ps, double jgx, double jgy, double xf, double yf,
+    const Consts<double>& K, Macro<double>& m)
+{
+    node_macro_dp<true>(ph, ps, jgx, jgy, xf, yf, K, m);
+}
+
+// Interface quantities of one node for the interface lattice alone (interface_flux).
+template <>
+__device__ __forceinline__ void interface_flux<double>(const Win<double>& ph,
+                                                       const Consts<double>& K, double& jx,
+                                                       double& jy)
+{
+    double gx, gy;
+    grad12(ph, gx, gy);
+    const double gm = sqrt(fmad(gx, gx, gy * gy));
+    const double ig = rcp_(gm + 12e-6);
+    const double theta_m = K.F.sharp * (ph.c * (1.0 - ph.c));
+    jx = theta_m * (gx * ig);
+    jy = theta_m * (gy * ig);
+}
+
+// Populations from the nine raw moments (raw_to_pop_fast); the factors 1/2 and 1/4 move into fmads.
+__device__ __forceinline__ void raw_to_pop_dp(double r00, double r10, double r01, double r20,
+                                              double r02, double r11, double r21, double r12,
+                                              double r22, double q[9])
+{
+    const double a = r20 - r22, b = r02 - r22;
+    const double sx = r10 - r12, sy = r01 - r21;
+    q[0] = (r00 - a) - (b + r22);   // (with b as rounded: the sum of the nine stays r00)
+    const double ha = 0.5 * a, hb = 0.5 * b;
+    q[1] = fmad(0.5, sx, ha);
+    q[3] = fmad(-0.5, sx, ha);
+    q[2] = fmad(0.5, sy, hb);
+    q[4] = fmad(-0.5, sy, hb);
+    const double qs = 0.25 * (r22 + r21), qt = 0.25 * (r22 - r21);
+    const double u = r11 + r12, v = r12 - r11;
+    q[5] = fmad(0.25, u, qs);
+    q[6] = fmad(-0.25, u, qs);
+    q[7] = fmad(-0.25, v, qt);
+    q[8] = fmad(0.25, v, qt);
+}
+
+// Fluid-lattice collision in double precision (collide_fluid).  The equilibrium is the Maxwellian
+// of density rho c^2 at u plus that of density p - rho c^2 at rest, so its raw moments about 0 are
+// products (rho c^2 (u_x^2 + 1/3) u_y and so on) and only the two relaxed central moments, al (half
+// the deviator's departure) and n11 keep, are shifted by u.
+template <>
+__device__ __forceinline__ void collide_fluid<double>(double g[9], double pstar,
+                                                      const Macro<double>& m)
+{
+    const double third = 1.0 / 3.0, ninth = 1.0 / 9.0, half = 0.5, two = 2.0;
+    const double ux = m.ux, uy = m.uy, mx = m.mx, my = m.my;
+    const double ux2 = ux * ux, uy2 = uy * uy, uxy = ux * uy;
+    const double rxx = mx * ux, ryy = my * uy, rxy = mx * uy;   // rho c^2 u u
+    // second-order raw moments of g-bar that survive the collision (deviator and 11)
+    const double dev = (g[1] + g[3]) - (g[2] + g[4]);
+    const double e11 = (g[5] - g[6]) + (g[7] - g[8]);
+    const double keep = 1.0 - m.omega, hk = half * keep;
+    const double al = hk * (dev - (rxx - ryy));
+    const double n11 = e11 - rxy, be2 = (two * keep) * n11;   // 2 be
+    // sources: sigma' (Gamma^t + Gamma^p matched, truncated), h-hat_0..2 and delta g^s, from
+    // (F_t + F_p) / 3 and H = F_p . u / 3
+    const double Fx = fmad(two, m.Ft6x, m.Fp3x), Fy = fmad(two, m.Ft6y, m.Fp3y);
+    const double s11 = fmad(Fx, uy, Fy * ux);
+    const double hy = Fy * uy, al2 = fmad(hk, fmad(Fx, ux, -hy), al);
+    const double base = fmad(two, m.H, third * pstar);
+    const double r20 = (base + fmad(Fx, ux, rxx)) + al2;
+    const double r02 = (base + fmad(Fy, uy, ryy)) - al2;
+    // (the source enters with 1 - omega / 2)
+    const double r11 = fmad(fmad(half, keep, half), s11, fmad(keep, n11, rxy));
+    double r21 = fmad(my, fmad(ux, ux, third), 2.0 / 3.0 * m.Ft6y);
+    double r12 = fmad(mx, fmad(uy, uy, third), 2.0 / 3.0 * m.Ft6x);
+    r21 = fmad(uy, al, fmad(ux, be2, r21));
+    r12 = fmad(ux, -al, fmad(uy, be2, r12));
+    double r22 = fmad(third, ryy, fmad(5.0 / 6.0, m.H, ninth * pstar));
+    r22 = fmad(rxx, uy2, fmad(third, rxx, r22));
+    r22 = fmad(uy2 - ux2, al, fmad(two * uxy, be2, r22));
+    const double r00 = fmad(3.0, m.H, pstar);
+    raw_to_pop_dp(r00, mx + m.Ft6x, my + m.Ft6y, r20, r02, r11, r21, r12, r22, g);
+}
+
+// Interface-lattice collision in double precision (collide_ace).
+template <>
+__device__ __forceinline__ void collide_ace<double>(double f[9], double phi,
+                                                    const Macro<double>& m, double omega_phi)
+{
+    const double third = 1.0 / 3.0, ninth = 1.0 / 9.0, two = 2.0;
+    const double ux = m.ux, uy = m.uy;
+    const double ux2 = ux * ux, uy2 = uy * uy;
+    double k10, k01;
+    first_moments(f, k10, k01);
+    const double keep = 1.0 - omega_phi;
+    const double mphi = -phi;
+    // a = c10 + omega (M_phi theta n_x - c10) with c10 = k10 - ux phi
+    const double a = fmad(keep, fmad(mphi, ux, k10), m.jx);
+    const double b = fmad(keep, fmad(mphi, uy, k01), m.jy);
+    const double cp = third * phi;
+    const double r10 = fmad(ux, phi, a);
+    const double r01 = fmad(uy, phi, b);
+    const double r20 = fmad(ux, r10 + a, cp);
+    const double r02 = fmad(uy, r01 + b, cp);
+    const double r11 = fmad(uy, r10, ux * b);
+    const double bx2 = ux2 * b;
+    const double r21 = fmad(uy, r20, bx2);
+    const double r12 = fmad(ux, r02, uy2 * a);
+    const double r22 = fmad(uy2, r20, fmad(two * uy, bx2, fmad(ux2, cp, ninth * phi)));
+    raw_to_pop_dp(phi, r10, r01, r20, r02, r11, r21, r12, r22, f);
 }
 
 // Populations from the nine raw moments (00,10,01,20,02,11,21,12,22) of D2Q9, closed form.

@@ -228,6 +228,18 @@ Consts<R> make_consts(const lbm_params& P)
     K.u0pi = R(P.u0 * 3.14159265358979323846);
     K.inv_nx = R(1.0 / P.nx);
     K.inv_ny = R(1.0 / P.ny);
+    if constexpr (std::is_same<R, double>::value) {
+        K.F.mu3_b = 3.0 * P.mu_b;
+        K.F.dmu3 = 3.0 * (P.mu_a - P.mu_b);
+        K.F.kt0 = 1.5 * P.width * P.sigma0 / 864.0;
+        K.F.dktx = 1.5 * P.width * P.dsigma_dT * P.gradT_x / 864.0;
+        K.F.dkty = 1.5 * P.width * P.dsigma_dT * P.gradT_y / 864.0;
+        K.F.sharp = P.mobility * 4.0 / P.width / (3.0 * P.mobility + 0.5);
+        K.F.gx = P.gx / 6.0;
+        K.F.gy = P.gy / 6.0;
+        K.F.cs2_drho = (P.rho_a - P.rho_b) / 108.0;
+        K.F.forces = P.gx != 0 || P.gy != 0 || K.dktx != 0 || K.dkty != 0 ? 1 : 0;
+    }
     return K;
 }
 

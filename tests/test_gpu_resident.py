@@ -123,6 +123,24 @@ def test_resident_batch_variants(collision, sigma_model):
         assert np.array_equal(ga, gb) and np.array_equal(fa, fb)
 
 
+@pytest.mark.parametrize("n", [2, 7, 30, 45])
+def test_resident_batches_of_a_few_waves(n):
+    """Counts for which the waves' blocks stay below the tallest that fit (30, 45) or not."""
+    rng = np.random.default_rng(n)
+    cases = [W.random_drop(int(rng.integers(32, 257)), int(rng.integers(32, 257)), seed=i,
+                           rho_ratio=100.0) for i in range(n)]
+    outs = []
+    for resident in (True, False):
+        with lbm.Batch(cases, precision="fp32") as b:
+            b.init_all()
+            if not resident:
+                lbm.lbm_batch_set_persistent(b.b, 0)
+            b.step(33)
+            outs.append([b.populations(i) for i in range(n)])
+    for (ga, fa), (gb, fb) in zip(*outs):
+        assert np.array_equal(ga, gb) and np.array_equal(fa, fb)
+
+
 def test_grids_beyond_shared_memory_and_of_one_node_take_the_other_forms():
     for nx, ny in ((1, 30), (30, 1), (700, 900)):
         case = W.random_drop(nx, ny, seed=4, wall_y=1, rho_ratio=10.0)

@@ -14,7 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libcmlbm.so")
 SOURCES = ["lbm_step.cu", "lbm_api.cu", "lbm_batch.cu", "lbm_resident.cu"]
-HEADERS = ["lbm_device.cuh", "lbm_host.h", "lbm_resident.h"]
+HEADERS = ["lbm_device.cuh", "lbm_host.h", "lbm_resident.h", "lbm_resident_rules.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
               "-I", os.path.join(ROOT, "include")]

@@ -63,6 +63,48 @@ def test_resident_runs_match_single_steps(nx, ny, bx, by, precision):
     assert np.array_equal(a[0], b[0])
 
 
+# grids of blocks that take two rounds of 16 rows (27, 17 = 16 + 1, 22 rows), beside no-slip and
+# free-slip sides: the first row of the second round is pushed into from both
+@pytest.mark.parametrize("precision", ["fp32", "fp16", "bf16"])
+@pytest.mark.parametrize("nx,ny,bx,by", [
+    (512, 512, (1, 1), (0, 0)),
+    (256, 640, (1, 1), (1, 1)),
+    (256, 640, (1, 2), (2, 1)),
+    (256, 640, (2, 1), (1, 2)),
+    (320, 640, (2, 2), (1, 1)),
+])
+def test_rounds_beside_side_walls(nx, ny, bx, by, precision):
+    test_resident_runs_match_single_steps(nx, ny, bx, by, precision)
+
+
+@pytest.mark.parametrize("bx", [(1, 1), (1, 2)])
+def test_three_rounds_beside_side_walls(bx):
+    """Blocks of 35 rows; and with the interface lattice alone of 43 rows."""
+    test_resident_runs_match_single_steps(128, 2600, bx, (1, 1), "fp32")
+    case = W.shear_circle(L0=640, u0=0.03)
+    case.update(wall_x=bx[0], wall_x_hi=bx[1])
+    out = [run(case, "fp32", r, (17, 33))[0].view(np.float32).reshape(640, -1, 18, 32)[:, :, 9:]
+           for r in (True, False)]
+    assert np.array_equal(out[0], out[1])
+
+
+def test_rounds_of_a_batch_beside_side_walls():
+    cases = [W.random_drop(nx, ny, seed=nx, wall_x=bx, wall_x_hi=hi, wall_y=1, rho_ratio=50.0,
+                           gravity=1e-6)
+             for nx, ny, bx, hi in ((200, 220, 1, 1), (90, 250, 1, 2), (130, 180, 2, 1))] * 12
+    for precision in ("fp32", "fp16"):
+        outs = []
+        for resident in (True, False):
+            with lbm.Batch(cases, precision=precision, layout=lbm.LBM_BATCH_AS_GIVEN) as b:
+                b.init_all()
+                if not resident:
+                    lbm.lbm_batch_set_persistent(b.b, 0)
+                b.step(65)
+                outs.append([b.populations(i) for i in range(len(cases))])
+        for (ga, fa), (gb, fb) in zip(*outs):
+            assert np.array_equal(ga, gb) and np.array_equal(fa, fb)
+
+
 @pytest.mark.parametrize("ny", [66, 900])
 @pytest.mark.parametrize("collision,sigma_model", [(1, 0), (0, 1), (1, 1)])
 def test_resident_step_variants(collision, sigma_model, ny):

@@ -42,9 +42,7 @@
 // between the polls (no gain).
 #include "lbm_device.cuh"
 #include "lbm_resident.h"
-#include "lbm_resident_rules.h"
 
-#include <algorithm>
 #include <type_traits>
 #include <vector>
 
@@ -1097,76 +1095,6 @@ cudaError_t launch_resident(void* state, const Geometry& G, const Consts<float>&
                                        args, P.Z.smem, st);
 }
 
-// Waves of a batch: every case gets the fewest blocks of at most `cap` rows; cases of like block
-// heights share a wave (its step takes as long as its tallest block), and the blocks a wave has left
-// go to the cases with its tallest.
-struct WavePart {
-    int c, nstrip, nseg, h;
-};
-static std::vector<std::vector<WavePart>> waves_of(const Geometry* G, int ncases, int nsm, int cap)
-{
-    std::vector<WavePart> parts;
-    for (int c = 0; c < ncases; ++c) {
-        WavePart p = {c, (G[c].nx + 63) / 64, (G[c].ny + cap - 1) / cap, 0};
-        p.h = (G[c].ny + p.nseg - 1) / p.nseg;
-        if (p.nstrip * p.nseg > nsm) return {};
-        parts.push_back(p);
-    }
-    std::stable_sort(parts.begin(), parts.end(),
-                     [](const WavePart& a, const WavePart& b) { return a.h > b.h; });
-    std::vector<std::vector<WavePart>> bins;
-    std::vector<int> used;
-    for (const WavePart& p : parts) {
-        size_t w = 0;
-        while (w < bins.size() && used[w] + p.nstrip * p.nseg > nsm) ++w;
-        if (w == bins.size()) {
-            bins.push_back({});
-            used.push_back(0);
-        }
-        bins[w].push_back(p);
-        used[w] += p.nstrip * p.nseg;
-    }
-    for (size_t w = 0; w < bins.size(); ++w) {
-        std::vector<WavePart>& b = bins[w];
-        for (;;) {
-            WavePart* t = &b[0];
-            for (WavePart& p : b)
-                if (p.h > t->h) t = &p;
-            // one segment more at a time shortens the tallest only now and then: go to the next
-            // count that does
-            int n = t->nseg + 1;
-            while (n <= G[t->c].ny / 2 && (G[t->c].ny + n - 1) / n == t->h) ++n;
-            if (n > G[t->c].ny / 2 || used[w] + (n - t->nseg) * t->nstrip > nsm) break;
-            used[w] += (n - t->nseg) * t->nstrip;
-            t->nseg = n;
-            t->h = (G[t->c].ny + n - 1) / n;
-        }
-    }
-    return bins;
-}
-
-static int tallest(const std::vector<WavePart>& wave)
-{
-    int h = 2;
-    for (const WavePart& p : wave) h = std::max(h, p.h);
-    return h;
-}
-
-// A step of a wave, in units of one row for each of four warps: the exchange and the sums (kStepRows),
-// the rows of the tallest block by fours (a warp of each quarter SM), and the start of every further
-// round of 16.  One GB300, FP32, us a step of blocks of 8, 12, 16, 20, 24, 28, 32, 36 rows (all SMs,
-// 4 strips): 3.2, 3.4, 3.9, 4.6, 5.1, 5.6, 6.3, 7.0; FP16 up to 32: 3.8, 4.5, 5.2, 6.5, 6.9, 7.6, 8.2.
-static double step_cost(int h)
-{
-    constexpr double kStepRows = 4.5, kRound = 0.6;
-    return kStepRows + (h + 3) / 4 + kRound * ((h + NW - 1) / NW - 1);
-}
-
-// The taller its blocks, the less of a step a wave spends in the exchange; but a batch short of
-// several full waves goes faster in one more wave of lower ones than in a last wave nearly empty.
-// The block height cap with the shortest sum over the waves is taken (multiples of four, and what
-// fits).  One GB300, FP32 drops of sides 32 - 256, us a step, always what fits / this: 30 cases 17.1 /
-// 15.5, 45 25.0 / 23.8, 140 81.3 / 79.8; 16, 24, 64, 100 and 192 keep the same plan.
 template <typename S, int V>
 bool resident_batch_plan(const Geometry* G, int ncases, int nsm, std::vector<ResidentWave>* waves)
 {
@@ -1176,21 +1104,11 @@ bool resident_batch_plan(const Geometry* G, int ncases, int nsm, std::vector<Res
     if (fit < 2) return false;
     for (int c = 0; c < ncases; ++c)
         if (!grid_splits<V>(G[c], (G[c].nx + 63) / 64)) return false;
-    std::vector<std::vector<WavePart>> bins = waves_of(G, ncases, nsm, fit);
-    if (bins.empty()) return false;
-    auto cost = [](const std::vector<std::vector<WavePart>>& b) {
-        double t = 0;
-        for (const auto& wave : b) t += step_cost(tallest(wave));
-        return t;
-    };
-    double best = cost(bins);
-    for (int cap = 8; cap < fit; cap += 4) {
-        std::vector<std::vector<WavePart>> other = waves_of(G, ncases, nsm, cap);
-        if (other.empty() || cost(other) >= best) continue;
-        best = cost(other);
-        bins.swap(other);
-    }
-    for (const std::vector<WavePart>& b : bins) {
+    std::vector<GridSize> grids;
+    for (int c = 0; c < ncases; ++c) grids.push_back({G[c].nx, G[c].ny});
+    const std::vector<Wave> plan = batch_waves(grids, nsm, fit);
+    if (plan.empty()) return false;
+    for (const Wave& b : plan) {
         ResidentWave W;
         int nblocks = 0;
         for (const WavePart& p : b) {

@@ -6,10 +6,9 @@
 #include <vector>
 
 #include "lbm_device.cuh"
+#include "lbm_resident_rules.h"
 
 namespace cmlbm {
-
-constexpr int kResidentWarps = 16;   // warps of a block; one block per SM
 
 // A grid's blocks: nstrip strips of 64 columns times nseg row segments, numbered from block0.
 struct ResidentGrid {
@@ -73,8 +72,8 @@ cudaError_t launch_resident(void* state, const Geometry&, const Consts<float>&,
                             const ResidentPlan&, int nsteps, int flow_sign, unsigned tag0,
                             void* box, void* lists, int* err, cudaStream_t);
 
-// The same for a batch, one launch per wave; false where a case does not fit.  The waves of a
-// batch may share one set of mailboxes (zeroed by the caller), with tags that continue from launch
+// The same for a batch, one launch per wave, the wave of the most blocks first; false where a case
+// does not fit.  The waves of a batch may share one set of mailboxes (zeroed by the caller), with tags that continue from launch
 // to launch; case_of[b] is the index into `cases` of block b of the wave.
 template <typename S, int V>
 bool resident_batch_plan(const Geometry*, int ncases, int nsm, std::vector<ResidentWave>*);

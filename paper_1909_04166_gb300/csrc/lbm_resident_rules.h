@@ -2,6 +2,9 @@
 // the kernel, its launches and the CPU tests share.
 #pragma once
 
+#include <algorithm>
+#include <vector>
+
 #ifdef __CUDACC__
 #define CMLBM_RULE __host__ __device__ __forceinline__
 #else
@@ -9,6 +12,8 @@
 #endif
 
 namespace cmlbm {
+
+constexpr int kResidentWarps = 16;   // warps of a block; one block per SM
 
 // The carry row holds what the last row of a round pushed north, planes 2, 5 and 6 of the row above
 // it, which the next round, whose first row that is, copies into place while it pushes.  Two words of
@@ -20,6 +25,121 @@ CMLBM_RULE bool carry_fills(int plane, int column, int width, bool noslip_left, 
 {
     return !(noslip_left && plane == 5 && column == 0) &&
            !(noslip_right && plane == 6 && column == width - 1);
+}
+
+// ---- plans ----------------------------------------------------------------------------------
+struct GridSize {
+    int nx, ny;
+};
+
+// A step of a launch, in units of one row for each of four warps: the exchange and the sums
+// (kStepRows), the rows of the tallest block by fours (a warp of each quarter SM), and the start of
+// every further round of 16.  One GB300, FP32, us a step of blocks of 2, 4, 8, 12, 16, 20, 24, 28, 32,
+// 36 rows (all SMs, 4 strips): 2.6, 2.8, 3.3, 3.5, 4.0, 4.8, 5.3, 5.8, 6.5, 7.3; FP16 up to 32: 3.0,
+// 3.3, 3.8, 4.6, 5.3, 6.6, 7.1, 7.7, 8.4.
+inline double step_cost(int h)
+{
+    constexpr double kStepRows = 4.5, kRound = 0.6;
+    return kStepRows + (h + 3) / 4 + kRound * ((h + kResidentWarps - 1) / kResidentWarps - 1);
+}
+
+// Waves of a batch: every case gets the fewest blocks of at most `cap` rows; cases of like block
+// heights share a wave (its step takes as long as its tallest block), and the blocks a wave has left
+// go to the cases with its tallest.
+struct WavePart {
+    int c, nstrip, nseg, h;
+};
+using Wave = std::vector<WavePart>;
+
+inline int tallest(const Wave& wave)
+{
+    int h = 2;
+    for (const WavePart& p : wave) h = std::max(h, p.h);
+    return h;
+}
+inline int blocks_of(const Wave& wave)
+{
+    int n = 0;
+    for (const WavePart& p : wave) n += p.nstrip * p.nseg;
+    return n;
+}
+inline double waves_cost(const std::vector<Wave>& waves)
+{
+    double t = 0;
+    for (const Wave& wave : waves) t += step_cost(tallest(wave));
+    return t;
+}
+
+inline std::vector<Wave> waves_of(const std::vector<GridSize>& G, int nsm, int cap)
+{
+    std::vector<WavePart> parts;
+    int smallest = nsm;
+    for (int c = 0; c < (int)G.size(); ++c) {
+        WavePart p = {c, (G[c].nx + 63) / 64, (G[c].ny + cap - 1) / cap, 0};
+        p.h = (G[c].ny + p.nseg - 1) / p.nseg;
+        if (p.nstrip * p.nseg > nsm) return {};
+        smallest = std::min(smallest, p.nstrip * p.nseg);
+        parts.push_back(p);
+    }
+    std::stable_sort(parts.begin(), parts.end(),
+                     [](const WavePart& a, const WavePart& b) { return a.h > b.h; });
+    std::vector<Wave> bins;
+    std::vector<int> used;
+    size_t open = 0;   // first wave that could still take a case
+    for (const WavePart& p : parts) {
+        while (open < bins.size() && used[open] + smallest > nsm) ++open;
+        size_t w = open;
+        while (w < bins.size() && used[w] + p.nstrip * p.nseg > nsm) ++w;
+        if (w == bins.size()) {
+            bins.push_back({});
+            used.push_back(0);
+        }
+        bins[w].push_back(p);
+        used[w] += p.nstrip * p.nseg;
+    }
+    for (size_t w = 0; w < bins.size(); ++w) {
+        Wave& b = bins[w];
+        for (;;) {
+            WavePart* t = &b[0];
+            for (WavePart& p : b)
+                if (p.h > t->h) t = &p;
+            // one segment more at a time shortens the tallest only now and then: go to the next
+            // count that does
+            int n = t->nseg + 1;
+            while (n <= G[t->c].ny / 2 && (G[t->c].ny + n - 1) / n == t->h) ++n;
+            if (n > G[t->c].ny / 2 || used[w] + (n - t->nseg) * t->nstrip > nsm) break;
+            used[w] += (n - t->nseg) * t->nstrip;
+            t->nseg = n;
+            t->h = (G[t->c].ny + n - 1) / n;
+        }
+    }
+    return bins;
+}
+
+// The taller its blocks, the less of a step a wave spends in the exchange; but a batch short of
+// several full waves goes faster in one more wave of lower ones than in a last wave nearly empty.
+// The block height cap with the shortest sum over the waves is taken (multiples of four, and what
+// fits).  One GB300, FP32 drops of sides 32 - 256, us a step, always what fits / this: 30 cases 17.1 /
+// 15.5, 45 25.0 / 23.8, 140 81.3 / 79.8; 16, 24, 64, 100 and 192 keep the same plan.
+//
+// The wave of the most blocks comes first: a device (or a part of one) on which not all its blocks
+// can be resident refuses its launch, so that a run is either refused before any case has moved, or
+// not at all.  Empty where a case does not fit.
+inline std::vector<Wave> batch_waves(const std::vector<GridSize>& G, int nsm, int fit)
+{
+    std::vector<Wave> best = waves_of(G, nsm, fit);
+    if (best.empty()) return best;
+    double least = waves_cost(best);
+    for (int cap = 8; cap < fit; cap += 4) {
+        std::vector<Wave> other = waves_of(G, nsm, cap);
+        if (other.empty() || waves_cost(other) >= least) continue;
+        least = waves_cost(other);
+        best.swap(other);
+    }
+    std::stable_sort(best.begin(), best.end(), [](const Wave& a, const Wave& b) {
+        return blocks_of(a) > blocks_of(b);
+    });
+    return best;
 }
 
 }  // namespace cmlbm

@@ -1,6 +1,7 @@
 """The rules of the resident kernel that need no GPU (csrc/lbm_resident_rules.h), compiled here as
 plain C++ and held against what the scheme does."""
 import os
+import random
 import subprocess
 
 import pytest
@@ -12,13 +13,14 @@ EX = (0, 1, 0, -1, 0, 1, -1, -1, 1)
 EY = (0, 0, 1, 0, -1, 1, 1, -1, -1)
 
 
-def compiled(tmp_path, body):
+def compiled(tmp_path, body, stdin=""):
     """Run a C++ program `body` that includes the rules; its output lines, split."""
     src, exe = tmp_path / "rules.cpp", tmp_path / "rules"
     src.write_text('#include <cstdio>\n#include "lbm_resident_rules.h"\nusing namespace cmlbm;\n'
                    + body)
     subprocess.run(["g++", "-std=c++17", "-O1", "-I", CSRC, "-o", str(exe), str(src)], check=True)
-    out = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout
+    out = subprocess.run([str(exe)], input=stdin, check=True, capture_output=True,
+                         text=True).stdout
     return [line.split() for line in out.splitlines()]
 
 
@@ -68,3 +70,40 @@ int main() {{
                     assert not 0 <= c < width or not 0 <= c - EX[a] < width
                     assert not (c == 0 and left == 1 and a == 5)
                     assert not (c == width - 1 and right == 1 and a == 6)
+
+
+PLAN = """
+int main() {
+    int nsm, fit, nx, ny;
+    std::vector<GridSize> G;
+    if (std::scanf("%d %d", &nsm, &fit) != 2) return 1;
+    while (std::scanf("%d %d", &nx, &ny) == 2) G.push_back({nx, ny});
+    for (const Wave& w : batch_waves(G, nsm, fit)) {
+        for (const WavePart& p : w) std::printf("%d %d %d %d ", p.c, p.nstrip, p.nseg, p.h);
+        std::printf("\\n");
+    }
+}"""
+
+
+@pytest.mark.parametrize("n,lo,hi", [(1, 2, 3), (5, 2, 700), (30, 32, 256), (192, 32, 256),
+                                     (300, 2, 64), (60, 300, 500)])
+@pytest.mark.parametrize("fit", [32, 36])
+def test_waves_hold_every_case_once_and_the_largest_comes_first(tmp_path, n, lo, hi, fit):
+    """A launch that the device refuses has to be the first one of a run: the waves come in
+    descending numbers of blocks."""
+    rng = random.Random(n * fit + hi)
+    grids = [(rng.randint(lo, hi), rng.randint(lo, hi)) for _ in range(n)]
+    src = f"152 {fit}\n" + "\n".join(f"{x} {y}" for x, y in grids)
+    waves = [[tuple(map(int, w[i:i + 4])) for i in range(0, len(w), 4)]
+             for w in compiled(tmp_path, PLAN, src)]
+    if any(-(-x // 64) * -(-y // fit) > 152 for x, y in grids):
+        assert not waves
+        return
+    assert sorted(c for w in waves for c, *_ in w) == list(range(n))
+    for w in waves:
+        for c, nstrip, nseg, h in w:
+            nx, ny = grids[c]
+            assert nstrip == -(-nx // 64) and h == -(-ny // nseg) <= fit
+            assert ny // nseg >= 2 or ny < 2
+    blocks = [sum(nstrip * nseg for _, nstrip, nseg, _ in w) for w in waves]
+    assert blocks == sorted(blocks, reverse=True) and blocks[0] <= 152

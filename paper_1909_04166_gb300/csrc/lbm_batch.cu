@@ -320,9 +320,9 @@ bool with_resident(const lbm_batch* b, F&& f)
 }
 
 // Make the waves, allocate what they need and fill it; false if a case does not fit or the
-// memory is not there.
+// memory, the host's included, is not there (no exception may leave the C entry points).
 bool plan_resident(lbm_batch* b)
-{
+try {
     const int n = (int)b->cases.size();
     std::vector<Geometry> G;
     for (const HostCase& hc : b->cases) G.push_back(hc.G);
@@ -380,6 +380,9 @@ bool plan_resident(lbm_batch* b)
         });
     }
     return e == cudaSuccess;
+} catch (const std::bad_alloc&) {
+    b->waves.clear();
+    return false;
 }
 
 // The resident kernel takes a run: allowed (no launch form or shape of the caller's), long

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <algorithm>
+#include <new>
 #include <vector>
 
 #ifdef __CUDACC__
@@ -124,9 +125,9 @@ inline std::vector<Wave> waves_of(const std::vector<GridSize>& G, int nsm, int c
 //
 // The wave of the most blocks comes first: a device (or a part of one) on which not all its blocks
 // can be resident refuses its launch, so that a run is either refused before any case has moved, or
-// not at all.  Empty where a case does not fit.
+// not at all.  Empty where a case does not fit or host memory runs out.
 inline std::vector<Wave> batch_waves(const std::vector<GridSize>& G, int nsm, int fit)
-{
+try {
     std::vector<Wave> best = waves_of(G, nsm, fit);
     if (best.empty()) return best;
     double least = waves_cost(best);
@@ -140,6 +141,8 @@ inline std::vector<Wave> batch_waves(const std::vector<GridSize>& G, int nsm, in
         return blocks_of(a) > blocks_of(b);
     });
     return best;
+} catch (const std::bad_alloc&) {
+    return {};
 }
 
 }  // namespace cmlbm

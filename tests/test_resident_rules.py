@@ -107,3 +107,38 @@ def test_waves_hold_every_case_once_and_the_largest_comes_first(tmp_path, n, lo,
             assert ny // nseg >= 2 or ny < 2
     blocks = [sum(nstrip * nseg for _, nstrip, nseg, _ in w) for w in waves]
     assert blocks == sorted(blocks, reverse=True) and blocks[0] <= 152
+
+
+def test_a_plan_without_host_memory_is_no_plan(tmp_path):
+    """Whichever allocation fails while a batch is planned, the plan is empty and nothing is thrown
+    (the plan is made inside a C entry point)."""
+    out = compiled(tmp_path, """
+#include <cstdlib>
+static int left = -1;
+void* operator new(std::size_t n)
+{
+    if (left == 0) throw std::bad_alloc();
+    if (left > 0) --left;
+    return std::malloc(n);
+}
+void operator delete(void* p) noexcept { std::free(p); }
+void operator delete(void* p, std::size_t) noexcept { std::free(p); }
+int main()
+{
+    std::vector<GridSize> G;
+    for (int i = 0; i < 40; ++i) G.push_back({40 + 5 * i, 250 - 3 * i});
+    const size_t all = batch_waves(G, 152, 36).size();
+    int failed = 0;
+    for (int k = 0;; ++k) {
+        left = k;
+        const size_t n = batch_waves(G, 152, 36).size();
+        const bool ran_out = left == 0;
+        left = -1;
+        if (!ran_out || n == all) break;
+        if (n != 0) return 1;
+        ++failed;
+    }
+    std::printf("%d %d\\n", failed, (int)all);
+}""")
+    failed, waves = map(int, out[0])
+    assert failed > 20 and waves > 1

@@ -1,8 +1,9 @@
 """Throughput of the fused cascaded two-phase LB step on GB300.
 
 One bench step = one time step of both D2Q9 lattices over the whole grid; the timed steps are
-one launch of the multi-step kernel, or one fused kernel launch per step where lbm_step takes
-graph replays (the line names the kernel, its launches and the form).  Default workload: drop
+one launch of the resident kernel (grids held in shared memory) or of the multi-step kernel, or one
+fused kernel launch per step where lbm_step takes graph replays (the line names the kernel, its
+launches and the form).  Default workload: drop
 impact on a thin film at density ratio 1000 on a 2048 x 1024 grid (the paper's Sec. 6.6
 parameters at Re = 100, We = 8000), FP32 populations (the bandwidth headline).  Prints one JSON
 line.
@@ -39,7 +40,6 @@ STORAGE = {"fp32": "FP32 populations", "fp64": "FP64 populations",
 HBM_FALLBACK_GBS = 6800.0
 L2_BYTES = 129e6
 METRIC = "MLUPS (million node updates of both lattices per second)"
-MULTI_MAX_STEPS = 65536     # steps per launch of the multi-step kernel (lbm_step splits longer runs)
 
 
 def workload(name: str):
@@ -81,7 +81,7 @@ def measured_peak():
 
 def kernel_source_hash() -> str:
     h = hashlib.sha256()
-    for f in ("lbm_step.cu", "lbm_device.cuh"):
+    for f in ("lbm_step.cu", "lbm_device.cuh", "lbm_resident.cu", "lbm_resident_rules.h"):
         with open(os.path.join(ROOT, "paper_1909_04166_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -219,12 +219,12 @@ def run_ours(args):
     dev = {k: torch.tensor(fl[k], dtype=torch.float64, device="cuda") for k in
            ("phi", "p", "ux", "uy")}
     lbm.lbm_init_fields_device(ctx, *(dev[k].data_ptr() for k in ("phi", "p", "ux", "uy")))
-    path = lbm.lbm_get_step_path(ctx)
     clk = Clocks(local, "warm-up, timed region and e2e leg").__enter__()
     lbm.lbm_step(ctx, args.warmup)
     torch.cuda.synchronize()
 
     K = args.steps
+    path, launches = lbm.lbm_get_run_path(ctx, K)   # every launch in the region is a step kernel
     ev0 = torch.cuda.Event(enable_timing=True)
     ev1 = torch.cuda.Event(enable_timing=True)
     if ws > 1:
@@ -232,16 +232,12 @@ def run_ours(args):
     torch.cuda.synchronize()
     queue_behind_spin(stream)
     ev0.record(stream)
-    lbm.lbm_step(ctx, K)             # one multi-step launch, or K graph-replayed launches
+    lbm.lbm_step(ctx, K)             # one launch, or K graph-replayed ones
     ev1.record(stream)
     torch.cuda.synchronize()
     if ws > 1:
         dist.barrier()
     ms_total = ev0.elapsed_time(ev1)
-    # every launch in the region is the step kernel: K launches, or ceil(K / 65536) launches of
-    # the multi-step kernel (each of up to 65536 steps)
-    multi = K >= 2 and path == lbm.LBM_PATH_MULTI
-    launches = -(-K // MULTI_MAX_STEPS) if multi else K
     ms_launch = ms_total / launches
     ms_max = max_over_ranks(ms_total, ws)
     diag = lbm.lbm_diagnostics(ctx)
@@ -284,16 +280,22 @@ def run_ours(args):
     achieved = bpl * N * steps_per_launch / (ms_launch * 1e-3) / 1e9
     traffic = None
     hsh = kernel_source_hash()
-    key = (hsh, args.workload, args.precision, "multi" if multi else "step")
+    narrow = "_narrow" if args.precision in ("fp16", "bf16") else ""
+    form, kname, how = {
+        lbm.LBM_PATH_RESIDENT: ("resident", "cmlbm::resident_kernel",
+                                "one cooperative launch of the resident kernel per run (state in "
+                                "shared memory, waits only between neighbouring blocks)"),
+        lbm.LBM_PATH_MULTI: ("multi", "cmlbm::step_kernel_multi" + narrow,
+                             "one cooperative launch of the multi-step kernel per run (waits only "
+                             "between neighbouring warps)"),
+    }.get(path, ("step", "cmlbm::step_kernel" + narrow,
+                 "graph replays of one step-kernel launch per step"))
+    key = (hsh, args.workload, args.precision, form)
     if key in NCU_TRAFFIC:   # DRAM bytes per step, for this launch's steps
         traffic = int(round(NCU_TRAFFIC[key] * steps_per_launch))
-    if multi:
-        kname = "cmlbm::step_kernel_multi" + ("_narrow" if args.precision in ("fp16", "bf16")
-                                              else "")
-    else:
-        kname = ("cmlbm::step_kernel_narrow" if args.precision in ("fp16", "bf16")
-                 else "cmlbm::step_kernel")
-    seg, block = None, None
+    # the resident kernel reads and writes the state once a launch: no share of the HBM rate then
+    # says how near the kernel is to its bound
+    resident = path == lbm.LBM_PATH_RESIDENT
     value = job_mlups(ws, N, K, ms_max)
     line = {
         "metric": METRIC,
@@ -310,8 +312,9 @@ def run_ours(args):
         "data": "synthetic (seeded initial fields of the paper's setup; no dataset)",
         "config": line_config(args, case, ws),
         "roofline": {
-            "bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
-            "frac": round(achieved / peak, 4), "traffic": traffic,
+            "bound": "exchange latency and FP32 issue" if resident else "hbm",
+            "achieved": None if resident else round(achieved, 1), "peak": peak, "unit": "GB/s",
+            "frac": None if resident else round(achieved / peak, 4), "traffic": traffic,
             "peak_source": f"{peak_kind} HBM copy bandwidth",
             "bytes_per_lu": bpl, "ms_per_launch": round(ms_launch, 5),
             "steps_per_launch": round(steps_per_launch, 3),
@@ -320,9 +323,7 @@ def run_ours(args):
         "clocks": clk.summary(),
         "e2e": e2e,
         "gpu_launches": launches,
-        "step_path": ("one cooperative launch of the multi-step kernel per run (waits only "
-                      "between neighbouring warps)" if multi else
-                      "graph replays of one step-kernel launch per step"),
+        "step_path": how,
         "state_check": {"sum_phi": diag["sum_phi"], "max_speed": diag["max_speed"],
                         "nonfinite": diag["nonfinite"]},
     }
@@ -346,7 +347,8 @@ def run_ours(args):
 
 def measure_ensemble(steps, per_case_steps, precision="fp32", device=0, stream=0):
     """The 512-case batch of independent static / oscillating drops: aggregate MLUPS of the
-    batched launch (autotuned), and of the same cases advanced by one launch per case."""
+    batch (autotuned; the form that its run takes is named), and of the same cases advanced by one
+    launch per case."""
     import torch
 
     from paper_1909_04166_gb300 import lbm
@@ -359,6 +361,8 @@ def measure_ensemble(steps, per_case_steps, precision="fp32", device=0, stream=0
         b.init_all()
         seg, block = lbm.lbm_batch_tune(b.b, 4)
         b.step(8)
+        path, launches = lbm.lbm_batch_get_run_path(b.b, steps)
+        resident = path == lbm.LBM_PATH_RESIDENT
         torch.cuda.synchronize()
         e0 = torch.cuda.Event(enable_timing=True)
         e1 = torch.cuda.Event(enable_timing=True)
@@ -370,9 +374,15 @@ def measure_ensemble(steps, per_case_steps, precision="fp32", device=0, stream=0
         lbm.lbm_batch_check(b.b)
         out.update({"batched_mlups": round(total * steps / (ms * 1e-3) / 1e6, 1),
                     "batched_ms_per_step": round(ms / steps, 4), "steps": steps,
-                    "tuned_launch": {"seg_rows": seg, "block": block},
-                    "batched_gbs": round(BYTES_PER_LU[precision] * total * steps / (ms * 1e-3)
-                                         / 1e9, 1)})
+                    "kernel": "cmlbm::resident_batch_kernel" if resident else
+                              "cmlbm::batch_step_kernel" + ("_narrow" if precision in
+                                                            ("fp16", "bf16") else ""),
+                    "launches": launches,
+                    # the launch shape of runs that the resident kernel does not take, and their
+                    # algorithmic traffic: neither says anything of a resident run
+                    "tuned_launch": None if resident else {"seg_rows": seg, "block": block},
+                    "batched_gbs": None if resident else
+                    round(BYTES_PER_LU[precision] * total * steps / (ms * 1e-3) / 1e9, 1)})
     if per_case_steps > 0:
         sims = [lbm.Simulation(c, precision=precision, device=device, stream=stream)
                 for c in cases]
@@ -633,13 +643,15 @@ def run_ensemble_line(args):
         "data": "synthetic (seeded ensemble of drop cases; no dataset)",
         "config": {"workload": f"ensemble of {r['cases']} drop cases, {r['nodes']} nodes, "
                                f"{args.precision} populations", "nodes": r["nodes"]},
-        "roofline": {"bound": "hbm", "achieved": r["batched_gbs"], "peak": peak, "unit": "GB/s",
-                     "frac": round(r["batched_gbs"] / peak, 4),
+        "roofline": {"bound": "hbm" if r["batched_gbs"] else "exchange latency and FP32 issue",
+                     "achieved": r["batched_gbs"], "peak": peak, "unit": "GB/s",
+                     "frac": r["batched_gbs"] and round(r["batched_gbs"] / peak, 4),
                      "traffic": NCU_TRAFFIC.get((kernel_source_hash(), "ensemble",
-                                                 args.precision, "step")),
+                                                 args.precision,
+                                                 "step" if r["batched_gbs"] else "resident")),
                      "peak_source": f"{peak_kind} HBM copy bandwidth",
-                     "kernel": "cmlbm::batch_step_kernel"},
-        "clocks": clk.summary(), "ensemble": r, "gpu_launches": args.steps,
+                     "kernel": r["kernel"]},
+        "clocks": clk.summary(), "ensemble": r, "gpu_launches": r["launches"],
     }
     print(json.dumps(line), flush=True)
 

@@ -248,8 +248,21 @@ int lbm_set_persistent(lbm_ctx* ctx, int32_t enable);
  * LBM_PATH_MULTI (one multi-step launch), LBM_PATH_GRAPHS (graph replays of one launch per step)
  * or LBM_PATH_SINGLE (one launch per step: graphs off, the bounds-checked kernel, or the first-
  * wait timeout injection).  LBM_ERR_ARG for NULL arguments. */
-enum { LBM_PATH_SINGLE = 0, LBM_PATH_GRAPHS = 1, LBM_PATH_MULTI = 2 };
+enum { LBM_PATH_SINGLE = 0, LBM_PATH_GRAPHS = 1, LBM_PATH_MULTI = 2, LBM_PATH_RESIDENT = 3 };
 int lbm_get_step_path(lbm_ctx* ctx, int32_t* path);
+
+/* How lbm_step would advance nsteps (>= 1) steps now.  *path: the form of its (first) run, which is
+ * LBM_PATH_RESIDENT where the resident kernel takes it, else what lbm_get_step_path says for two or
+ * more steps and LBM_PATH_SINGLE for one.  *launches: the step kernels that all of it launches (one a
+ * step in the graphs); NULL allowed.  May make the plan and allocate the buffers that such a call
+ * itself would.  LBM_ERR_ARG for NULL or nsteps < 1. */
+int lbm_get_run_path(lbm_ctx* ctx, int32_t nsteps, int32_t* path, int32_t* launches);
+
+/* The resident kernel of lbm_step: enable = 1 (default) lets it take the runs described there, 0 keeps
+ * them from it.  It leaves the other forms' settings alone, so that enable = 1 also takes back what
+ * lbm_set_persistent 0 or 1 and lbm_set_launch say about the resident kernel.  Results are identical.
+ * Other values: LBM_ERR_ARG. */
+int lbm_set_resident(lbm_ctx* ctx, int32_t enable);
 
 /* Debugging aid standing in for a memory checker: run the following steps through a variant of
  * the step kernel that checks every global load, store and bulk copy of a step against the
@@ -445,6 +458,10 @@ int lbm_batch_get_launch(const lbm_batch* b, int32_t* seg_rows, int32_t* block_t
  * LBM_PATH_GRAPHS. */
 int lbm_batch_set_persistent(lbm_batch* b, int32_t enable);
 int lbm_batch_get_step_path(const lbm_batch* b, int32_t* path);
+
+/* As lbm_get_run_path and lbm_set_resident, for a batch. */
+int lbm_batch_get_run_path(lbm_batch* b, int32_t nsteps, int32_t* path, int32_t* launches);
+int lbm_batch_set_resident(lbm_batch* b, int32_t enable);
 
 /* Autotuner: times trial_steps (>= 1) steps of the live batch for each candidate launch shape
  * (rows per task 8..64, blocks of 64 or 128 threads), keeps the fastest and restores the state

@@ -295,6 +295,14 @@ int flow_sign_at(const lbm_ctx* c, long long t)
     return (c->P.reverse_step > 0 && t >= c->P.reverse_step) ? -1 : 1;
 }
 
+// How many of nsteps steps from time level t a run takes: those until the imposed flow reverses (its
+// sign is constant within a run).
+long long run_of(const lbm_ctx* c, long long t, long long nsteps)
+{
+    if (flow_sign_at(c, t) <= 0 || c->P.reverse_step <= 0) return nsteps;
+    return std::min<long long>(nsteps, c->P.reverse_step - t);
+}
+
 cudaError_t launch_one(lbm_ctx* c, const void* src, void* dst, int sign)
 {
     if (c->checked) {
@@ -693,11 +701,8 @@ int lbm_step(lbm_ctx* c, int32_t nsteps)
     if (!c->initialised) return LBM_ERR_STATE;
     int32_t k = 0;
     while (k < nsteps) {
-        // steps until the imposed flow reverses (the sign is constant within a run)
         const int sign = flow_sign_at(c, c->steps);
-        long long run = nsteps - k;
-        if (sign > 0 && c->P.reverse_step > 0)
-            run = std::min<long long>(run, c->P.reverse_step - c->steps);
+        long long run = run_of(c, c->steps, nsteps - k);
         while (resident_takes(c, run)) {   // in place: the current buffer is unchanged
             const int chunk = (int)std::min<long long>(run, kMultiMaxSteps);
             cudaError_t e = launch_resident_run(c, chunk, sign);
@@ -767,6 +772,38 @@ int lbm_get_step_path(lbm_ctx* c, int32_t* path)
     if (multi_fits(c)) *path = LBM_PATH_MULTI;
     else if (c->use_graph && !c->checked && !c->cut_first_wait) *path = LBM_PATH_GRAPHS;
     else *path = LBM_PATH_SINGLE;
+    return LBM_OK;
+}
+
+int lbm_get_run_path(lbm_ctx* c, int32_t nsteps, int32_t* path, int32_t* launches)
+{
+    if (!c || !path || nsteps < 1) return LBM_ERR_ARG;
+    int32_t rest = LBM_PATH_SINGLE, first = -1;
+    lbm_get_step_path(c, &rest);
+    long long n = 0, t = c->steps;
+    for (long long left = nsteps; left > 0;) {   // the choices of lbm_step
+        long long run = run_of(c, t, left);
+        left -= run;
+        t += run;
+        while (resident_takes(c, run)) {
+            if (first < 0) first = LBM_PATH_RESIDENT;
+            run -= std::min<long long>(run, kMultiMaxSteps);
+            ++n;
+        }
+        if (first < 0) first = run >= 2 ? rest : LBM_PATH_SINGLE;
+        if (rest == LBM_PATH_MULTI)
+            for (; run >= 2; ++n) run -= std::min<long long>(run, kMultiMaxSteps);
+        n += run;
+    }
+    *path = first;
+    if (launches) *launches = (int32_t)n;
+    return LBM_OK;
+}
+
+int lbm_set_resident(lbm_ctx* c, int32_t enable)
+{
+    if (!c || enable < 0 || enable > 1) return LBM_ERR_ARG;
+    c->use_resident = enable;
     return LBM_OK;
 }
 

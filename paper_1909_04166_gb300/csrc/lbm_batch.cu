@@ -15,6 +15,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <new>
 #include <type_traits>
 #include <utility>
@@ -32,6 +33,8 @@ namespace {
 // runs of n >= 2 steps replay graphs of an even number of steps, 2 .. 32 (32-step graphs while at
 // least 32 steps are left, then one for the even rest; the parity returns after each)
 constexpr int kBatchGraphSizes = 16;
+// steps of one launch of the kernels that take more than one
+constexpr int kMaxSteps = 1 << 16;
 
 struct HostCase {
     lbm_params P;           // as stored: the reflected problem when tr
@@ -559,7 +562,7 @@ int lbm_batch_step(lbm_batch* b, int32_t nsteps)
     cudaSetDevice(b->device);
     int32_t k = 0;
     while (resident_takes(b, nsteps - k)) {   // in place: the parity is unchanged
-        const int chunk = std::min(nsteps - k, 1 << 16);
+        const int chunk = std::min(nsteps - k, kMaxSteps);
         cudaError_t e = cudaSuccess;
         for (size_t w = 0; w < b->waves.size() && e == cudaSuccess; ++w) {
             e = launch_resident_wave(b, w, chunk);
@@ -573,8 +576,8 @@ int lbm_batch_step(lbm_batch* b, int32_t nsteps)
         }
         k += chunk;
     }
-    while (nsteps - k >= 2 && multi_fits(b)) {   // one multi-step launch per 65536 steps
-        const int chunk = std::min(nsteps - k, 1 << 16);
+    while (nsteps - k >= 2 && multi_fits(b)) {   // one multi-step launch per kMaxSteps steps
+        const int chunk = std::min(nsteps - k, kMaxSteps);
         cudaError_t e = launch_multi_run(b, chunk);
         if (e != cudaSuccess) return fail_cuda(b, e);
         k += chunk;
@@ -678,6 +681,35 @@ int lbm_batch_get_step_path(const lbm_batch* b, int32_t* path)
 {
     if (!b || !path) return LBM_ERR_ARG;
     *path = multi_fits(b) ? LBM_PATH_MULTI : LBM_PATH_GRAPHS;
+    return LBM_OK;
+}
+
+int lbm_batch_get_run_path(lbm_batch* b, int32_t nsteps, int32_t* path, int32_t* launches)
+{
+    if (!b || !path || nsteps < 1) return LBM_ERR_ARG;
+    cudaSetDevice(b->device);
+    int32_t first = -1;
+    int run = nsteps;
+    long long n = 0;
+    while (resident_takes(b, run)) {   // the choices of lbm_batch_step
+        first = LBM_PATH_RESIDENT;
+        run -= std::min(run, kMaxSteps);
+        n += (long long)b->waves.size();
+    }
+    const bool multi = multi_fits(b);
+    if (first < 0) first = run < 2 ? LBM_PATH_SINGLE : multi ? LBM_PATH_MULTI : LBM_PATH_GRAPHS;
+    if (multi)
+        for (; run >= 2; ++n) run -= std::min(run, kMaxSteps);
+    n += run;
+    *path = first;
+    if (launches) *launches = (int32_t)std::min<long long>(n, INT32_MAX);
+    return LBM_OK;
+}
+
+int lbm_batch_set_resident(lbm_batch* b, int32_t enable)
+{
+    if (!b || enable < 0 || enable > 1) return LBM_ERR_ARG;
+    b->use_resident = enable;
     return LBM_OK;
 }
 

@@ -57,7 +57,8 @@ EXPORTS = [
     "lbm_batch_get_populations", "lbm_batch_set_launch", "lbm_batch_get_launch",
     "lbm_batch_tune", "lbm_batch_nodes", "lbm_batch_check", "lbm_batch_destroy",
     "lbm_batch_create_ex", "lbm_batch_case_transposed", "lbm_batch_set_persistent",
-    "lbm_batch_get_step_path",
+    "lbm_batch_get_step_path", "lbm_get_run_path", "lbm_set_resident",
+    "lbm_batch_get_run_path", "lbm_batch_set_resident",
 ]
 
 
@@ -142,6 +143,8 @@ def lib(build_if_missing: bool = True):
     L.lbm_set_graphs.argtypes = [vp, i32]
     L.lbm_set_persistent.argtypes = [vp, i32]
     L.lbm_get_step_path.argtypes = [vp, P(i32)]
+    L.lbm_get_run_path.argtypes = [vp, i32, P(i32), P(i32)]
+    L.lbm_set_resident.argtypes = [vp, i32]
     L.lbm_set_checked.argtypes = [vp, i32]
     L.lbm_inject_timeout.argtypes = [vp, i32]
     dd = ctypes.c_double
@@ -158,6 +161,8 @@ def lib(build_if_missing: bool = True):
     L.lbm_batch_get_launch.argtypes = [vp, P(i32), P(i32)]
     L.lbm_batch_set_persistent.argtypes = [vp, i32]
     L.lbm_batch_get_step_path.argtypes = [vp, P(i32)]
+    L.lbm_batch_get_run_path.argtypes = [vp, i32, P(i32), P(i32)]
+    L.lbm_batch_set_resident.argtypes = [vp, i32]
     L.lbm_batch_tune.argtypes = [vp, i32, P(i32), P(i32)]
     L.lbm_batch_nodes.argtypes = [vp]
     L.lbm_batch_nodes.restype = i64
@@ -300,13 +305,26 @@ def lbm_set_persistent(ctx, enable) -> None:
     _check(lib().lbm_set_persistent(ctx, int(enable)), "lbm_set_persistent")
 
 
-LBM_PATH_SINGLE, LBM_PATH_GRAPHS, LBM_PATH_MULTI = 0, 1, 2
+LBM_PATH_SINGLE, LBM_PATH_GRAPHS, LBM_PATH_MULTI, LBM_PATH_RESIDENT = 0, 1, 2, 3
 
 
 def lbm_get_step_path(ctx) -> int:
     v = ctypes.c_int32()
     _check(lib().lbm_get_step_path(ctx, ctypes.byref(v)), "lbm_get_step_path")
     return int(v.value)
+
+
+def lbm_get_run_path(ctx, nsteps: int):
+    """(form of the run, step kernels it launches) of nsteps steps issued now."""
+    path, launches = ctypes.c_int32(), ctypes.c_int32()
+    _check(lib().lbm_get_run_path(ctx, int(nsteps), ctypes.byref(path), ctypes.byref(launches)),
+           "lbm_get_run_path")
+    return int(path.value), int(launches.value)
+
+
+def lbm_set_resident(ctx, enable) -> None:
+    """True / 1: the resident kernel takes the runs it can; False / 0: never."""
+    _check(lib().lbm_set_resident(ctx, int(enable)), "lbm_set_resident")
 
 
 def lbm_set_checked(ctx, enable) -> None:
@@ -417,6 +435,18 @@ def lbm_batch_get_step_path(b) -> int:
     v = ctypes.c_int32()
     _check(lib().lbm_batch_get_step_path(b, ctypes.byref(v)), "lbm_batch_get_step_path")
     return int(v.value)
+
+
+def lbm_batch_get_run_path(b, nsteps: int):
+    """(form of the run, step kernels it launches) of nsteps steps issued now."""
+    path, launches = ctypes.c_int32(), ctypes.c_int32()
+    _check(lib().lbm_batch_get_run_path(b, int(nsteps), ctypes.byref(path), ctypes.byref(launches)),
+           "lbm_batch_get_run_path")
+    return int(path.value), int(launches.value)
+
+
+def lbm_batch_set_resident(b, enable) -> None:
+    _check(lib().lbm_batch_set_resident(b, int(enable)), "lbm_batch_set_resident")
 
 
 def lbm_batch_tune(b, trial_steps: int = 8):

@@ -191,3 +191,71 @@ def test_grids_beyond_shared_memory_and_of_one_node_take_the_other_forms():
             before = lbm.lbm_state_device(sim.ctx)[0]
             sim.step(17)
             assert lbm.lbm_state_device(sim.ctx)[0] != before
+
+
+def test_run_paths_name_the_form_that_runs_take():
+    """lbm_get_run_path against where a run leaves the state (in place: resident), for run lengths,
+    after each setting that keeps runs from the resident kernel and after lbm_set_resident."""
+    case = W.random_drop(70, 60, seed=9, rho_ratio=10.0)
+    with lbm.Simulation(case, precision="fp32") as sim:
+        sim.init_case()
+
+        def check(n, resident, launches=None):
+            path, count = lbm.lbm_get_run_path(sim.ctx, n)
+            before = lbm.lbm_state_device(sim.ctx)[0]
+            sim.step(n)
+            assert (lbm.lbm_state_device(sim.ctx)[0] == before) == resident
+            assert (path == lbm.LBM_PATH_RESIDENT) == resident
+            assert launches is None or count == launches
+
+        check(17, True, 1)
+        check(15, False, 15)
+        check(1, False, 1)
+        for keep, back in ((lambda: lbm.lbm_set_persistent(sim.ctx, 0), None),
+                           (lambda: lbm.lbm_set_launch(sim.ctx, 4, 0), None),
+                           (lambda: lbm.lbm_set_resident(sim.ctx, 0), None),
+                           (lambda: lbm.lbm_set_graphs(sim.ctx, 0),
+                            lambda: lbm.lbm_set_graphs(sim.ctx, 1))):
+            keep()
+            check(17, False, 17)
+            if back:
+                back()
+            lbm.lbm_set_resident(sim.ctx, 1)
+            check(17, True, 1)
+        lbm.lbm_set_persistent(sim.ctx, 1)
+        assert lbm.lbm_get_run_path(sim.ctx, 17) == (lbm.LBM_PATH_MULTI, 1)
+        for bad in (0, -3):
+            with pytest.raises(lbm.LbmError):
+                lbm.lbm_get_run_path(sim.ctx, bad)
+        for bad in (2, -1):
+            with pytest.raises(lbm.LbmError):
+                lbm.lbm_set_resident(sim.ctx, bad)
+    flow = W.shear_circle(L0=64, u0=0.03)
+    flow.update(reverse_step=20)
+    with lbm.Simulation(flow, precision="fp32") as sim:   # 20 steps, then 20 in the other direction
+        sim.init_case()
+        assert lbm.lbm_get_run_path(sim.ctx, 40) == (lbm.LBM_PATH_RESIDENT, 2)
+        assert lbm.lbm_get_run_path(sim.ctx, 25) == (lbm.LBM_PATH_RESIDENT, 1 + 5)
+
+
+def test_run_paths_of_a_batch():
+    cases = W.ensemble(6)
+    with lbm.Batch(cases, precision="fp32") as b:
+        b.init_all()
+        path, waves = lbm.lbm_batch_get_run_path(b.b, 40)
+        assert path == lbm.LBM_PATH_RESIDENT and 1 <= waves <= 6
+        assert lbm.lbm_batch_get_run_path(b.b, 15) == (lbm.LBM_PATH_GRAPHS, 15)
+        assert lbm.lbm_batch_get_run_path(b.b, 1) == (lbm.LBM_PATH_SINGLE, 1)
+        for keep in (lambda: lbm.lbm_batch_set_persistent(b.b, 0),
+                     lambda: lbm.lbm_batch_set_launch(b.b, 8, 0),
+                     lambda: lbm.lbm_batch_set_resident(b.b, 0)):
+            keep()
+            assert lbm.lbm_batch_get_run_path(b.b, 40) == (lbm.LBM_PATH_GRAPHS, 40)
+            lbm.lbm_batch_set_resident(b.b, 1)
+            assert lbm.lbm_batch_get_run_path(b.b, 40) == (path, waves)
+        lbm.lbm_batch_set_persistent(b.b, 1)
+        assert lbm.lbm_batch_get_run_path(b.b, 40) == (lbm.LBM_PATH_MULTI, 1)
+        with pytest.raises(lbm.LbmError):
+            lbm.lbm_batch_get_run_path(b.b, 0)
+        with pytest.raises(lbm.LbmError):
+            lbm.lbm_batch_set_resident(b.b, 2)

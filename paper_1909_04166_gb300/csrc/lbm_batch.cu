@@ -776,11 +776,11 @@ int lbm_batch_tune(lbm_batch* b, int32_t trial_steps, int32_t* seg_rows, int32_t
         cudaMemcpyAsync(b->base, backup, b->base_bytes, cudaMemcpyDeviceToDevice, b->st);
     if (e2 == cudaSuccess) e2 = cudaStreamSynchronize(b->st);
     cudaFree(backup);
+    if (e == cudaSuccess && e2 == cudaSuccess && !status)
+        status = lbm_batch_set_launch(b, best_seg, best_block);
+    b->use_resident = resident0;   // the tuner's shapes are for the runs it does not take
     if (e != cudaSuccess) return fail_cuda(b, e);
     if (e2 != cudaSuccess) return fail_cuda(b, e2);
-    if (status) return status;
-    status = lbm_batch_set_launch(b, best_seg, best_block);
-    b->use_resident = resident0;   // the tuner's shape is for the runs it does not take
     if (status) return status;
     if (seg_rows) *seg_rows = best_seg;
     if (block_threads) *block_threads = best_block;

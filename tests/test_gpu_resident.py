@@ -259,3 +259,23 @@ def test_run_paths_of_a_batch():
             lbm.lbm_batch_get_run_path(b.b, 0)
         with pytest.raises(lbm.LbmError):
             lbm.lbm_batch_set_resident(b.b, 2)
+
+
+def test_a_failed_tuning_leaves_the_resident_kernel_on():
+    """Tuning fails where it may not wait for the batch's stream: during a capture of it."""
+    import torch
+    stream = torch.cuda.Stream()
+    with lbm.Batch(W.ensemble(3), precision="fp32", stream=stream.cuda_stream) as b:
+        b.init_all()
+        assert lbm.lbm_batch_get_run_path(b.b, 40)[0] == lbm.LBM_PATH_RESIDENT
+        torch.cuda.synchronize()
+        with pytest.raises(Exception):
+            with torch.cuda.graph(torch.cuda.CUDAGraph(), stream=stream,
+                                  capture_error_mode="relaxed"):
+                try:
+                    lbm.lbm_batch_tune(b.b, 2)
+                    failed = False
+                except lbm.LbmError:
+                    failed = True
+        assert failed
+        assert lbm.lbm_batch_get_run_path(b.b, 40)[0] == lbm.LBM_PATH_RESIDENT

@@ -427,12 +427,14 @@ int lbm_batch_init_fields(lbm_batch* b, int32_t c, const double* phi, const doub
                           const double* ux, const double* uy);
 
 /* Advance every case by nsteps (>= 0) time steps; asynchronous on the batch's stream.  A run of
- * 16 or more steps (64 with 16-bit storage in large batches) of a batch with FP32 arithmetic whose
- * cases each fit the SMs' shared memory is issued as one launch of the resident kernel (lbm_step)
- * per wave, a set of cases that fit together, each launch taking its cases through all the steps;
- * the first such run allocates the message buffers (about 3 MB a wave).  If that fails, in a stream
- * capture, and once the caller has chosen a form or shape (lbm_batch_set_persistent,
- * lbm_batch_set_launch), runs take the other forms.  The results are the same, bit for bit. */
+ * 16 or more steps of a batch with FP32 arithmetic whose cases each fit the SMs' shared memory is
+ * issued, where that is faster than graph replays (every run of small batches; of large ones FP32 runs
+ * of more than about 40 steps, 16-bit runs of cases of few columns), as one launch of the resident
+ * kernel (lbm_step) per wave, a set of cases that fit together, each launch taking its cases through
+ * all the steps; the first such run allocates the message buffers (up to 18 MB for the batch, and about
+ * 3 MB a wave).  If that fails, in a stream capture, and once the caller has chosen a form or shape
+ * (lbm_batch_set_persistent, lbm_batch_set_launch), runs take the other forms.  The results are the
+ * same, bit for bit. */
 int lbm_batch_step(lbm_batch* b, int32_t nsteps);
 
 /* Fields / populations of case c, as lbm_get_fields / lbm_get_populations.  Synchronise. */
@@ -465,8 +467,8 @@ int lbm_batch_set_resident(lbm_batch* b, int32_t enable);
 
 /* Autotuner: times trial_steps (>= 1) steps of the live batch for each candidate launch shape
  * (rows per task 8..64, blocks of 64 or 128 threads), keeps the fastest and restores the state
- * it started from (a temporary device copy).  Which runs the resident kernel takes stays as it
- * was.  Synchronises. */
+ * it started from (a temporary device copy).  Runs that are faster with the resident kernel than
+ * the times found (lbm_batch_step) go on taking it.  Synchronises. */
 int lbm_batch_tune(lbm_batch* b, int32_t trial_steps, int32_t* seg_rows, int32_t* block_threads);
 
 /* Total nodes of all cases; LBM_ERR_TIMEOUT check as lbm_check; release (NULL allowed). */

@@ -104,6 +104,9 @@ struct lbm_batch {
     char* rmem;
     std::vector<size_t> wave_lists, wave_cases, wave_blocks;   // offsets in rmem
     unsigned rtag;          // tag of the last message sent
+    double waves_step;      // us a step of the waves and of graph replays, by which a run takes
+    double replays_step;    // the one or the other (replays: measured by a tuning, else modelled)
+    bool tuned;
 };
 
 namespace {
@@ -302,14 +305,8 @@ cudaError_t ensure_graphs(lbm_batch* b)
     return e;
 }
 
-// Shortest runs that go to the resident kernel, every wave of which is a launch that reads and
-// writes its part of the state once; 16-bit storage, whose steps gain less, in batches of more
-// than kBatchFewWaves waves only from kBatchResidentMinSteps16Bit on.  One GB300, us a step against
-// graph replays: 192 drops of sides 32 - 256 (18 waves), FP32, 16 steps 131 / 138, 1000 steps 107 /
-// 137; FP16, 32 steps 171 / 156, 64 steps 152 / 156, 1000 steps 143 / 155; 16 such drops (one or
-// two waves) 6.3 / 26 and 8.4 / 36.
-constexpr int kBatchResidentMinSteps = 16, kBatchResidentMinSteps16Bit = 64;
-constexpr size_t kBatchFewWaves = 2;
+// Shortest run that goes to the resident kernel (as in lbm_api.cu), if waves_pay says so as well.
+constexpr int kBatchResidentMinSteps = 16;
 
 // Call f(S{}, V{}) for the batch's storage and step variant where the resident kernel has them.
 template <class F>
@@ -330,9 +327,18 @@ try {
     std::vector<Geometry> G;
     for (const HostCase& hc : b->cases) G.push_back(hc.G);
     if (!with_resident(b, [&](auto s, auto v) {
-            return resident_batch_plan<decltype(s), decltype(v)::value>(G.data(), n, b->nsm,
-                                                                        &b->waves);
+            return resident_batch_plan<decltype(s), decltype(v)::value>(
+                G.data(), n, b->nsm, &b->waves, &b->waves_step);
         })) {
+        b->waves.clear();
+        return false;
+    }
+    if (!b->tuned) {
+        std::vector<GridSize> grids;
+        for (const Geometry& g : G) grids.push_back({g.nx, g.ny});
+        b->replays_step = replays_us(grids, b->precision != LBM_FP32);
+    }
+    if (b->waves_step >= b->replays_step) {   // no run would take them
         b->waves.clear();
         return false;
     }
@@ -389,7 +395,7 @@ try {
 }
 
 // The resident kernel takes a run: allowed (no launch form or shape of the caller's), long
-// enough, planned, and outside a stream capture (as in lbm_api.cu).
+// enough, planned, outside a stream capture (as in lbm_api.cu), and faster than graph replays.
 bool resident_takes(lbm_batch* b, int run)
 {
     if (!b->use_resident || b->resident_state < 0 || run < kBatchResidentMinSteps) return false;
@@ -400,9 +406,8 @@ bool resident_takes(lbm_batch* b, int run)
     }
     if (cap != cudaStreamCaptureStatusNone) return false;
     if (b->resident_state == 0) b->resident_state = plan_resident(b) ? 1 : -1;
-    const bool narrow = b->precision == LBM_FP32_FP16 || b->precision == LBM_FP32_BF16;
-    return b->resident_state == 1 && !(narrow && b->waves.size() > kBatchFewWaves &&
-                                       run < kBatchResidentMinSteps16Bit);
+    return b->resident_state == 1 &&
+           waves_pay(run, b->waves.size(), b->waves_step, b->replays_step);
 }
 
 cudaError_t launch_resident_wave(lbm_batch* b, size_t k, int nsteps)
@@ -776,8 +781,12 @@ int lbm_batch_tune(lbm_batch* b, int32_t trial_steps, int32_t* seg_rows, int32_t
         cudaMemcpyAsync(b->base, backup, b->base_bytes, cudaMemcpyDeviceToDevice, b->st);
     if (e2 == cudaSuccess) e2 = cudaStreamSynchronize(b->st);
     cudaFree(backup);
-    if (e == cudaSuccess && e2 == cudaSuccess && !status)
+    if (e == cudaSuccess && e2 == cudaSuccess && !status) {
         status = lbm_batch_set_launch(b, best_seg, best_block);
+        b->replays_step = 1e3 * best / trial_steps;
+        b->tuned = true;
+        if (b->resident_state < 0 && !b->rmem) b->resident_state = 0;   // plan by the time found
+    }
     b->use_resident = resident0;   // the tuner's shapes are for the runs it does not take
     if (e != cudaSuccess) return fail_cuda(b, e);
     if (e2 != cudaSuccess) return fail_cuda(b, e2);

@@ -1096,7 +1096,8 @@ cudaError_t launch_resident(void* state, const Geometry& G, const Consts<float>&
 }
 
 template <typename S, int V>
-bool resident_batch_plan(const Geometry* G, int ncases, int nsm, std::vector<ResidentWave>* waves)
+bool resident_batch_plan(const Geometry* G, int ncases, int nsm, std::vector<ResidentWave>* waves,
+                         double* step_us)
 {
     const int most = most_smem();
     int fit = 0;
@@ -1108,6 +1109,7 @@ bool resident_batch_plan(const Geometry* G, int ncases, int nsm, std::vector<Res
     for (int c = 0; c < ncases; ++c) grids.push_back({G[c].nx, G[c].ny});
     const std::vector<Wave> plan = batch_waves(grids, nsm, fit);
     if (plan.empty()) return false;
+    *step_us = waves_us(plan, Narrow<S>::value);
     for (const Wave& b : plan) {
         ResidentWave W;
         int nblocks = 0;
@@ -1153,7 +1155,7 @@ cudaError_t launch_resident_batch(void* base, const ResidentSizes& Z, const Resi
                                                void*, int*, cudaStream_t);
 #define CMLBM_INSTANTIATE_RESIDENT_BATCH(S, V)                                                    \
     template bool resident_batch_plan<S, V>(const Geometry*, int, int,                          \
-                                            std::vector<ResidentWave>*);                        \
+                                            std::vector<ResidentWave>*, double*);               \
     template cudaError_t prepare_resident_batch<S, V>(const ResidentSizes&,                     \
                                                       const ResidentCase*, const int*, void*,   \
                                                       cudaStream_t);                            \

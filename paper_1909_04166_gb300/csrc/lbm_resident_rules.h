@@ -145,4 +145,36 @@ try {
     return {};
 }
 
+// Whether a batch's run goes to the waves or to graph replays of one launch a step, from what either
+// takes.  Waves: kWaveUnit us a step for each unit of their cost, and kWaveRun us a wave and run, in
+// which it is launched and its part of the state read and written.  Replays of the default launch
+// shape: by the strips of 64 columns, filled or not, times their rows, and by the strips (whose last
+// segments are short).  One GB300, 96 - 2000 drops of sides 32 - 64, 32 - 256, 200 - 256 and 300 - 500
+// (1.8 - 20.7 million nodes): the waves' steps within 3 % of this, the replays' within 3 % in FP32
+// and 5 % in 16 bits (the waves are far ahead below that).  Measured, us a step, replays /
+// waves: FP32 192 drops 134 / 107, 512 311 / 264, 60 of sides 300 - 500 260 / 239 (in runs of 16
+// steps 286); FP16 192 drops 151 / 142, 512 340 / 351, 400 of sides 200 - 256 590 / 674, 2000 of
+// sides 32 - 64 189 / 182.
+constexpr double kWaveRun = 23.0;
+inline double wave_unit(bool narrow) { return narrow ? 0.638 : 0.495; }
+
+inline double waves_us(const std::vector<Wave>& waves, bool narrow)
+{
+    return wave_unit(narrow) * waves_cost(waves);
+}
+inline double replays_us(const std::vector<GridSize>& G, bool narrow)
+{
+    double nodes = 0, strips = 0;
+    for (const GridSize& g : G) {
+        strips += (g.nx + 63) / 64;
+        nodes += 64.0 * ((g.nx + 63) / 64) * g.ny;
+    }
+    return narrow ? 27.6 + 24.1e-6 * nodes + 0.0171 * strips
+                  : 18.2 + 22.4e-6 * nodes + 0.0188 * strips;
+}
+inline bool waves_pay(int steps, size_t nwaves, double waves_step, double replays_step)
+{
+    return steps * waves_step + kWaveRun * nwaves < steps * replays_step;
+}
+
 }  // namespace cmlbm

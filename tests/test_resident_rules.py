@@ -142,3 +142,90 @@ int main()
 }""")
     failed, waves = map(int, out[0])
     assert failed > 20 and waves > 1
+
+
+# drops, their sides, 16-bit storage, steps of a run; us a step measured on one GB300 as waves of the
+# resident kernel and as graph replays of the default launch shape
+MEASURED = [
+    (8, 32, 256, 0, 256, 4.7, 23.8),
+    (8, 32, 256, 0, 16, 5.7, 23.8),
+    (8, 32, 256, 1, 256, 6.2, 34.8),
+    (8, 32, 256, 1, 64, 6.4, 34.8),
+    (32, 32, 256, 0, 256, 18.0, 32.2),
+    (32, 32, 256, 0, 16, 21.5, 32.2),
+    (32, 32, 256, 1, 256, 23.9, 43.8),
+    (32, 32, 256, 1, 64, 24.6, 43.8),
+    (64, 32, 256, 0, 256, 34.2, 44.7),
+    (64, 32, 256, 0, 16, 41.3, 44.7),
+    (64, 32, 256, 1, 256, 46.2, 56.2),
+    (64, 32, 256, 1, 64, 47.7, 56.2),
+    (128, 32, 256, 0, 256, 65.9, 88.2),
+    (128, 32, 256, 0, 16, 79.2, 88.2),
+    (128, 32, 256, 1, 256, 86.4, 99.9),
+    (128, 32, 256, 1, 64, 89.2, 99.9),
+    (192, 32, 256, 0, 256, 107.0, 134.3),
+    (192, 32, 256, 0, 16, 128.6, 134.3),
+    (192, 32, 256, 1, 256, 142.4, 151.2),
+    (192, 32, 256, 1, 64, 147.1, 151.2),
+    (384, 32, 256, 0, 256, 198.7, 237.8),
+    (384, 32, 256, 0, 16, 237.8, 237.8),
+    (384, 32, 256, 1, 256, 265.1, 265.2),
+    (384, 32, 256, 1, 64, 273.8, 265.2),
+    (512, 32, 256, 0, 256, 263.7, 310.6),
+    (512, 32, 256, 0, 16, 315.9, 310.6),
+    (512, 32, 256, 1, 256, 351.3, 339.9),
+    (512, 32, 256, 1, 64, 362.8, 339.9),
+    (768, 32, 256, 0, 256, 379.5, 439.8),
+    (768, 32, 256, 0, 16, 454.4, 439.8),
+    (768, 32, 256, 1, 256, 506.4, 480.4),
+    (768, 32, 256, 1, 64, 522.9, 480.4),
+    (300, 32, 64, 0, 256, 21.2, 33.5),
+    (300, 32, 64, 0, 16, 25.2, 33.5),
+    (300, 32, 64, 1, 256, 28.7, 44.0),
+    (300, 32, 64, 1, 64, 29.5, 44.0),
+    (2000, 32, 64, 0, 256, 129.7, 178.5),
+    (2000, 32, 64, 0, 16, 156.4, 178.5),
+    (2000, 32, 64, 1, 256, 181.8, 189.4),
+    (2000, 32, 64, 1, 64, 187.5, 189.4),
+    (100, 200, 256, 0, 256, 126.8, 149.9),
+    (100, 200, 256, 0, 16, 151.7, 149.9),
+    (100, 200, 256, 1, 256, 167.5, 166.1),
+    (100, 200, 256, 1, 64, 173.1, 166.1),
+    (400, 200, 256, 0, 256, 512.6, 552.3),
+    (400, 200, 256, 0, 16, 611.6, 552.3),
+    (400, 200, 256, 1, 256, 673.5, 590.4),
+    (400, 200, 256, 1, 64, 695.2, 590.4),
+    (60, 300, 500, 0, 256, 238.5, 260.4),
+    (60, 300, 500, 0, 16, 285.7, 260.4),
+    (60, 300, 500, 1, 256, 336.9, 285.9),
+    (60, 300, 500, 1, 64, 347.6, 285.9),
+]
+
+
+def test_the_form_of_a_batch_is_the_faster_one(tmp_path):
+    """The choice between waves and graph replays against measured times of both: within 3 % of the
+    faster one."""
+    import numpy as np
+    src = ""
+    for n, lo, hi, narrow, steps, _, _ in MEASURED:
+        rng = np.random.default_rng(n + lo)
+        grids = [(int(rng.integers(lo, hi + 1)), int(rng.integers(lo, hi + 1))) for _ in range(n)]
+        src += f"{n} {32 if narrow else 36} {narrow} {steps}\n"
+        for x, y in grids:   # each stored in the orientation of fewer padded columns
+            src += "%d %d\n" % ((y, x) if -(-y // 64) * x < -(-x // 64) * y else (x, y))
+    out = compiled(tmp_path, """
+int main()
+{
+    int n, fit, narrow, steps;
+    while (std::scanf("%d %d %d %d", &n, &fit, &narrow, &steps) == 4) {
+        std::vector<GridSize> G(n);
+        for (GridSize& g : G)
+            if (std::scanf("%d %d", &g.nx, &g.ny) != 2) return 1;
+        const std::vector<Wave> w = batch_waves(G, 152, fit);
+        std::printf("%d\\n", (int)waves_pay(steps, w.size(), waves_us(w, narrow),
+                                            replays_us(G, narrow)));
+    }
+}""", src)
+    assert len(out) == len(MEASURED)
+    for (pays,), (*case, waves, replays) in zip(out, MEASURED):
+        assert (waves if pays == "1" else replays) <= 1.03 * min(waves, replays), case

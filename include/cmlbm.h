@@ -211,11 +211,14 @@ int lbm_init_fields_device(lbm_ctx* ctx, const double* phi, const double* p, con
  * asynchronous; launch errors are returned.  A run of 16 or more steps of a grid whose state the
  * SMs can hold in shared memory (FP32 arithmetic, up to about 350,000 nodes; the interface
  * lattice alone up to 650,000; 16-bit storage up to 310,000) is one launch of the resident
- * kernel: the state is read once, stays on the chip for the run (up to 65536 steps a launch),
- * and is written back in place.  Its first run allocates the message buffers (up to 30 MB) that
- * the blocks exchange their borders through; if that fails, in a stream capture, and with a
- * launch form or shape of the caller's (lbm_set_persistent 0 or 1, lbm_set_graphs 0,
- * lbm_set_launch) the forms below run instead.
+ * kernel: the state is read once, stays on the chip for the run (up to 4096 steps a launch), and is
+ * written back in place.  A context with a stream of its own (params.stream neither 0 nor
+ * cudaStreamLegacy) leaves room for others on other streams: its blocks take part of the device where
+ * several grids then run at once faster than one after another, and its runs the forms below where
+ * those share the device better (lbm_set_resident).  The kernel's first run allocates the message
+ * buffers (up to 30 MB) that the blocks exchange their borders through; if that fails, in a stream
+ * capture, and with a launch form or shape of the caller's (lbm_set_persistent 0 or 1, lbm_set_graphs
+ * 0, lbm_set_launch) the forms below run instead.
  * Otherwise a run of two or more steps is, where the multi-step
  * kernel is enabled (lbm_set_persistent; by default with LBM_FP32 storage where the warp
  * segments have at least 3 rows) and the grid's warps fit on the device at once, one launch of
@@ -259,9 +262,10 @@ int lbm_get_step_path(lbm_ctx* ctx, int32_t* path);
 int lbm_get_run_path(lbm_ctx* ctx, int32_t nsteps, int32_t* path, int32_t* launches);
 
 /* The resident kernel of lbm_step: enable = 1 (default) lets it take the runs described there, 0 keeps
- * them from it.  It leaves the other forms' settings alone, so that enable = 1 also takes back what
- * lbm_set_persistent 0 or 1 and lbm_set_launch say about the resident kernel.  Results are identical.
- * Other values: LBM_ERR_ARG. */
+ * them from it, 2 lets it take them with the whole device also on a stream of the context's own (for
+ * contexts that do not run side by side).  It leaves the other forms' settings alone, so that 1 and 2
+ * also take back what lbm_set_persistent 0 or 1 and lbm_set_launch say about the resident kernel.
+ * Results are identical.  Synchronises where the split changes.  Other values: LBM_ERR_ARG. */
 int lbm_set_resident(lbm_ctx* ctx, int32_t enable);
 
 /* Debugging aid standing in for a memory checker: run the following steps through a variant of
@@ -461,7 +465,7 @@ int lbm_batch_get_launch(const lbm_batch* b, int32_t* seg_rows, int32_t* block_t
 int lbm_batch_set_persistent(lbm_batch* b, int32_t enable);
 int lbm_batch_get_step_path(const lbm_batch* b, int32_t* path);
 
-/* As lbm_get_run_path and lbm_set_resident, for a batch. */
+/* As lbm_get_run_path and lbm_set_resident (0 and 1 only), for a batch. */
 int lbm_batch_get_run_path(lbm_batch* b, int32_t nsteps, int32_t* path, int32_t* launches);
 int lbm_batch_set_resident(lbm_batch* b, int32_t enable);
 

@@ -43,6 +43,7 @@ struct lbm_ctx {
     int use_multi;         // lbm_set_persistent
     int multi_bps;         // resident blocks per SM of the multi-step kernel (0: not usable)
     int use_resident;      // runs may go to the resident kernel (see resident_takes)
+    int whole_device;      // its plan takes the device for itself (lbm_set_resident 2)
     int resident_state;    // 0: no plan made yet, 1: plan and mailboxes ready, -1: not usable
     ResidentPlan rplan;
     void* box;             // its mailboxes, then its exchange lists
@@ -220,11 +221,18 @@ void* resident_lists(const lbm_ctx* c)
     return static_cast<char*>(c->box) + c->rplan.Z.box_bytes;
 }
 
+// Other contexts may run beside this one: it has a stream of its own (work on the default stream is
+// in one order).
+bool shares(const lbm_ctx* c)
+{
+    return !c->whole_device && c->st != nullptr && c->st != cudaStreamLegacy;
+}
+
 // The resident kernel takes a run: allowed (not with a launch form or shape chosen by the
 // caller, nor in a test or debugging mode), long enough, with a plan that fits, and outside a
 // stream capture (a captured launch would replay its message tags).  The plan is made and the
 // mailboxes allocated by the first run that could use them.  Wherever the state fits it was the
-// fastest form (lbm_resident.cu has the times).
+// fastest form of a grid by itself (lbm_resident.cu has the times).
 bool resident_takes(lbm_ctx* c, long long run)
 {
     if (!c->use_resident || !c->use_graph || c->checked || c->cut_first_wait ||
@@ -241,7 +249,8 @@ bool resident_takes(lbm_ctx* c, long long run)
         cudaSetDevice(c->P.device);
         const bool ok = with_variant(c->P.precision, c->variant, [&](auto r, auto s, auto v) {
             if constexpr (std::is_same<decltype(r), float>::value)
-                return resident_plan<decltype(s), decltype(v)::value>(c->G, c->nsm, &c->rplan);
+                return resident_plan<decltype(s), decltype(v)::value>(c->G, c->nsm, shares(c),
+                                                                      &c->rplan);
             else return false;
         });
         if (!ok) return false;
@@ -704,7 +713,7 @@ int lbm_step(lbm_ctx* c, int32_t nsteps)
         const int sign = flow_sign_at(c, c->steps);
         long long run = run_of(c, c->steps, nsteps - k);
         while (resident_takes(c, run)) {   // in place: the current buffer is unchanged
-            const int chunk = (int)std::min<long long>(run, kMultiMaxSteps);
+            const int chunk = (int)std::min<long long>(run, kResidentMaxSteps);
             cudaError_t e = launch_resident_run(c, chunk, sign);
             if (e == cudaErrorCooperativeLaunchTooLarge) {   // fewer SMs here than the device has
                 cudaGetLastError();
@@ -787,7 +796,7 @@ int lbm_get_run_path(lbm_ctx* c, int32_t nsteps, int32_t* path, int32_t* launche
         t += run;
         while (resident_takes(c, run)) {
             if (first < 0) first = LBM_PATH_RESIDENT;
-            run -= std::min<long long>(run, kMultiMaxSteps);
+            run -= std::min<long long>(run, kResidentMaxSteps);
             ++n;
         }
         if (first < 0) first = run >= 2 ? rest : LBM_PATH_SINGLE;
@@ -802,8 +811,19 @@ int lbm_get_run_path(lbm_ctx* c, int32_t nsteps, int32_t* path, int32_t* launche
 
 int lbm_set_resident(lbm_ctx* c, int32_t enable)
 {
-    if (!c || enable < 0 || enable > 1) return LBM_ERR_ARG;
-    c->use_resident = enable;
+    if (!c || enable < 0 || enable > 2) return LBM_ERR_ARG;
+    c->use_resident = enable != 0;
+    const bool before = shares(c);
+    if (enable) c->whole_device = enable == 2;
+    if (shares(c) != before && c->resident_state) {   // another plan: the next run makes it
+        cudaSetDevice(c->P.device);
+        cudaError_t e = cudaStreamSynchronize(c->st);
+        if (e != cudaSuccess) return cuda_fail(c, e);
+        cudaFree(c->box);
+        c->box = nullptr;
+        c->rtag = 0;
+        c->resident_state = 0;
+    }
     return LBM_OK;
 }
 

@@ -33,7 +33,7 @@ namespace {
 // runs of n >= 2 steps replay graphs of an even number of steps, 2 .. 32 (32-step graphs while at
 // least 32 steps are left, then one for the even rest; the parity returns after each)
 constexpr int kBatchGraphSizes = 16;
-// steps of one launch of the kernels that take more than one
+// steps of one launch of the multi-step kernel
 constexpr int kMaxSteps = 1 << 16;
 
 struct HostCase {
@@ -396,6 +396,10 @@ try {
 
 // The resident kernel takes a run: allowed (no launch form or shape of the caller's), long
 // enough, planned, outside a stream capture (as in lbm_api.cu), and faster than graph replays.
+// The waves take all SMs on any stream: batches are the way to run many cases at once, and several
+// side by side on eight streams still take no longer than their replays did (one GB300, us for a step
+// of all eight, waves / replays: of 2 drops FP32 19 / 29, 8 37 / 37, 16 77 / 77, FP16 26 / 38, 50 / 47),
+// but for FP16 batches of about 16 drops (104 / 85; one by itself 13 / 38).
 bool resident_takes(lbm_batch* b, int run)
 {
     if (!b->use_resident || b->resident_state < 0 || run < kBatchResidentMinSteps) return false;
@@ -567,7 +571,7 @@ int lbm_batch_step(lbm_batch* b, int32_t nsteps)
     cudaSetDevice(b->device);
     int32_t k = 0;
     while (resident_takes(b, nsteps - k)) {   // in place: the parity is unchanged
-        const int chunk = std::min(nsteps - k, kMaxSteps);
+        const int chunk = std::min(nsteps - k, kResidentMaxSteps);
         cudaError_t e = cudaSuccess;
         for (size_t w = 0; w < b->waves.size() && e == cudaSuccess; ++w) {
             e = launch_resident_wave(b, w, chunk);
@@ -698,7 +702,7 @@ int lbm_batch_get_run_path(lbm_batch* b, int32_t nsteps, int32_t* path, int32_t*
     long long n = 0;
     while (resident_takes(b, run)) {   // the choices of lbm_batch_step
         first = LBM_PATH_RESIDENT;
-        run -= std::min(run, kMaxSteps);
+        run -= std::min(run, kResidentMaxSteps);
         n += (long long)b->waves.size();
     }
     const bool multi = multi_fits(b);

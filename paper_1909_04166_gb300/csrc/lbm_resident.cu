@@ -1056,14 +1056,26 @@ ResidentLaunch launch_args(const ResidentSizes& z, void* box, void* lists, int n
 
 }  // namespace
 
+// Most rows of a block; 0 if not even two fit.
 template <typename S, int V>
-bool resident_plan(const Geometry& G, int nsm, ResidentPlan* out)
+int most_rows(int most)
 {
-    const int nstrip = (G.nx + 63) / 64;
+    int h = 0;
+    while (rows_fit<S, V>(h + 1, most)) ++h;
+    return h < 2 ? 0 : h;
+}
+
+template <typename S, int V>
+bool resident_plan(const Geometry& G, int nsm, bool shared, ResidentPlan* out)
+{
+    const int nstrip = (G.nx + 63) / 64, most = most_smem(), fit = most_rows<S, V>(most);
     if (!grid_splits<V>(G, nstrip) || nstrip > nsm) return false;
-    const int nseg = nsm / nstrip < G.ny / 2 ? nsm / nstrip : G.ny / 2;
-    const int hmax = (G.ny + nseg - 1) / nseg, most = most_smem();
-    if (!rows_fit<S, V>(hmax, most)) return false;
+    const GridSize size = {G.nx, G.ny};
+    constexpr Form form = (V & kVarShear) ? Form::Flow : Narrow<S>::value ? Form::Narrow : Form::Fp32;
+    const int nseg = shared ? shared_segments(size, nsm, fit, form) : most_segments(size, nsm);
+    if (nseg < 1) return false;
+    const int hmax = (G.ny + nseg - 1) / nseg;
+    if (hmax > fit) return false;
     out->D = {nstrip, nseg, 0};
     fill_sizes<S, V>(nstrip * nseg, hmax, &out->Z);
     return can_launch(resident_fn<S, V>(hmax), out->Z.smem, most);
@@ -1099,9 +1111,7 @@ template <typename S, int V>
 bool resident_batch_plan(const Geometry* G, int ncases, int nsm, std::vector<ResidentWave>* waves,
                          double* step_us)
 {
-    const int most = most_smem();
-    int fit = 0;
-    while (rows_fit<S, V>(fit + 1, most)) ++fit;
+    const int most = most_smem(), fit = most_rows<S, V>(most);
     if (fit < 2) return false;
     for (int c = 0; c < ncases; ++c)
         if (!grid_splits<V>(G[c], (G[c].nx + 63) / 64)) return false;
@@ -1147,7 +1157,7 @@ cudaError_t launch_resident_batch(void* base, const ResidentSizes& Z, const Resi
 }
 
 #define CMLBM_INSTANTIATE_RESIDENT(S, V)                                                          \
-    template bool resident_plan<S, V>(const Geometry&, int, ResidentPlan*);                     \
+    template bool resident_plan<S, V>(const Geometry&, int, bool, ResidentPlan*);               \
     template cudaError_t prepare_resident<S, V>(const Geometry&, const ResidentPlan&, void*,    \
                                                 void*, cudaStream_t);                           \
     template cudaError_t launch_resident<S, V>(void*, const Geometry&, const Consts<float>&,    \

@@ -55,10 +55,12 @@ struct ResidentLaunch {
     int* err;             // device error word (0 = ok)
 };
 
-// Plan for a grid on a device of nsm SMs (the current device); false where its state does not
-// fit in their shared memory, a block would have a single row, or the grid a single column.
+// Plan for a grid on a device of nsm SMs (the current device), with as many blocks as make a step
+// fastest by itself, or with shared, beside others on other streams (shared_segments); false where its
+// state does not fit in their shared memory, a block would have a single row, the grid a single
+// column, or shared_segments finds none.
 template <typename S, int V>
-bool resident_plan(const Geometry&, int nsm, ResidentPlan*);
+bool resident_plan(const Geometry&, int nsm, bool shared, ResidentPlan*);
 
 // Zero the caller's mailboxes (box_bytes) and fill its exchange lists (list_bytes), once per plan.
 template <typename S, int V>

@@ -177,4 +177,64 @@ inline bool waves_pay(int steps, size_t nwaves, double waves_step, double replay
     return steps * waves_step + kWaveRun * nwaves < steps * replays_step;
 }
 
+// A grid's segments.  Alone on the device a step is fastest over all SMs, each block a strip of 64
+// columns by as few rows as that leaves; but a block has its SM to itself, so that several contexts on
+// several streams then run one after another, where the small launches of graph replays ran side by
+// side.  A context on a stream of its own therefore takes the most segments (the lowest blocks, the
+// shortest step) with which neither it alone nor two, four or eight like it are slower than in the
+// other forms, and where there are none (0) the other forms.  Their times are modelled from one
+// GB300's: contexts alone, and eight side by side on eight streams.  All SMs / other forms / this, us
+// for a step of each of 1, 2, 4, 8 contexts:
+//   FP32 128 x 128   2.5 4.9 9.7 19.5 / 3.9 4.2 5.1 6.3 / 3.0 3.1 3.3 6.5
+//   FP32 256 x 256   3.3 6.6 13.1 26.4 / 5.3 6.9 9.6 19.7 / 4.0 4.0 8.1 16.0
+//   FP32 161 x 481   3.6 7.1 14.3 28.6 / 6.5 7.5 13.5 28.6 / 4.8 4.8 9.5 19.0
+//   BF16 512 x 256   5.1 10.2 20.4 40.8 / 7.8 10.3 16.4 33.1 / the other forms
+enum class Form { Fp32, Narrow, Flow };   // 32-bit and 16-bit storage; the interface lattice alone
+
+inline double resident_step_us(Form form, int h)   // blocks of h rows; within 8 % of the kernel's
+{
+    const int rounds = (h + kResidentWarps - 1) / kResidentWarps;
+    switch (form) {
+    case Form::Narrow: return 2.7 + 0.15 * h + 0.7 * (rounds - 1);
+    case Form::Flow: return 2.3 + 0.045 * h + 0.047 * std::max(0, h - 32);
+    default: return 2.35 + 0.115 * h + 0.35 * (rounds - 1);
+    }
+}
+struct OtherForms {
+    double alone, share;   // us a step of one by itself, and of each of many side by side
+};
+inline OtherForms other_forms(Form form, double nodes)   // (nodes of whole strips)
+{
+    switch (form) {
+    case Form::Narrow: return {4.2 + 27e-6 * nodes, 0.35 + 32e-6 * nodes};
+    case Form::Flow: return {3.5 + 14.5e-6 * nodes, 0.35 + 18e-6 * nodes};
+    default: return {3.4 + 31e-6 * nodes, 0.5 + 26e-6 * nodes};
+    }
+}
+inline int most_segments(GridSize G, int nsm)
+{
+    return std::min(nsm / ((G.nx + 63) / 64), G.ny / 2);
+}
+inline int shared_segments(GridSize G, int nsm, int fit, Form form)
+{
+    const int nstrip = (G.nx + 63) / 64;
+    const OtherForms other = other_forms(form, 64.0 * nstrip * G.ny);
+    for (int nseg = most_segments(G, nsm); nseg >= 1; --nseg) {
+        const int h = (G.ny + nseg - 1) / nseg;
+        const double step = resident_step_us(form, h);
+        if (h > fit || step > other.alone) break;
+        const int at_once = nsm / (nstrip * nseg);
+        bool no_slower = true;
+        for (int k = 2; k <= 8; k *= 2)
+            no_slower &= (k + at_once - 1) / at_once * step <= std::max(other.alone, k * other.share);
+        if (no_slower) return nseg;
+    }
+    return 0;
+}
+
+// Steps of one launch.  While it runs nobody else gets its SMs, so a longer run is cut: 4096 steps
+// take 10 - 35 ms, and what a launch costs beside its steps is 0.1 % of them or less (us a step in
+// launches of 512 / 4096 steps: 64 x 64 2.234 / 2.213, 400 x 700 7.190 / 7.148).
+constexpr int kResidentMaxSteps = 4096;
+
 }  // namespace cmlbm

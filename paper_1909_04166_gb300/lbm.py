@@ -323,7 +323,8 @@ def lbm_get_run_path(ctx, nsteps: int):
 
 
 def lbm_set_resident(ctx, enable) -> None:
-    """True / 1: the resident kernel takes the runs it can; False / 0: never."""
+    """True / 1: the resident kernel takes the runs it can; False / 0: never; 2: with the whole
+    device on any stream."""
     _check(lib().lbm_set_resident(ctx, int(enable)), "lbm_set_resident")
 
 

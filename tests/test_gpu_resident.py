@@ -227,7 +227,7 @@ def test_run_paths_name_the_form_that_runs_take():
         for bad in (0, -3):
             with pytest.raises(lbm.LbmError):
                 lbm.lbm_get_run_path(sim.ctx, bad)
-        for bad in (2, -1):
+        for bad in (3, -1):
             with pytest.raises(lbm.LbmError):
                 lbm.lbm_set_resident(sim.ctx, bad)
     flow = W.shear_circle(L0=64, u0=0.03)
@@ -279,3 +279,49 @@ def test_a_failed_tuning_leaves_the_resident_kernel_on():
                     failed = True
         assert failed
         assert lbm.lbm_batch_get_run_path(b.b, 40)[0] == lbm.LBM_PATH_RESIDENT
+
+
+def test_contexts_on_streams_of_their_own():
+    """Contexts side by side on five streams, four with a part of the device and one in the other
+    forms, over more than one launch's steps, against the whole device and against one launch per step on the default stream."""
+    import torch
+    shapes = ((64, 64, "fp32"), (130, 128, "fp32"), (200, 200, "bf16"), (161, 481, "fp32"),
+              (256, 256, "bf16"))
+    streams = [torch.cuda.Stream() for _ in shapes]
+    cases = [W.random_drop(nx, ny, seed=nx, wall_x=1, wall_y=2, rho_ratio=10.0) for nx, ny, _ in shapes]
+
+    def state(sim):
+        raw = sim.save_state()[0]
+        sim.close()
+        return raw
+
+    sims = [lbm.Simulation(c, precision=p, stream=s.cuda_stream)
+            for c, (_, _, p), s in zip(cases, shapes, streams)]
+    for sim in sims:
+        sim.init_case()
+        assert lbm.lbm_get_run_path(sim.ctx, 4120) == (
+            (lbm.LBM_PATH_GRAPHS, 4120) if sim.nx == 200 else (lbm.LBM_PATH_RESIDENT, 2))
+    for sim in sims:
+        sim.step(4120)
+    got = [state(sim) for sim in sims]
+    for i, (c, (_, _, p)) in enumerate(zip(cases, shapes)):
+        one = lbm.Simulation(c, precision=p).init_case()
+        lbm.lbm_set_resident(one.ctx, 0)
+        assert np.array_equal(got[i], state(one.step(4120)))
+        alone = lbm.Simulation(c, precision=p, stream=streams[i].cuda_stream).init_case().step(2000)
+        lbm.lbm_set_resident(alone.ctx, 2)     # another split for the rest of the run
+        alone.step(1100)
+        lbm.lbm_set_resident(alone.ctx, 1)
+        assert np.array_equal(got[i], state(alone.step(1020)))
+
+
+def test_a_grid_that_shares_the_device_better_in_the_other_forms():
+    import torch
+    case = W.random_drop(512, 256, seed=3, rho_ratio=10.0)
+    stream = torch.cuda.Stream()
+    with lbm.Simulation(case, precision="bf16", stream=stream.cuda_stream) as sim, \
+            lbm.Simulation(case, precision="bf16") as default:
+        assert lbm.lbm_get_run_path(sim.ctx, 40)[0] == lbm.LBM_PATH_GRAPHS
+        lbm.lbm_set_resident(sim.ctx, 2)
+        assert lbm.lbm_get_run_path(sim.ctx, 40)[0] == lbm.LBM_PATH_RESIDENT
+        assert lbm.lbm_get_run_path(default.ctx, 40)[0] == lbm.LBM_PATH_RESIDENT

@@ -180,7 +180,7 @@ __device__ __forceinline__ void upstream(const Geometry& G, const Block& B, int 
 // during a run.
 struct Lists {
     unsigned* node;          // row << 16 | column + 1 of the nodes of the two outermost rings
-    unsigned short* sdst;    // where a send goes: the neighbour (0 .. 7) << 13 | mailbox index
+    unsigned short* sdst;    // where a send goes: the neighbour's code << box_bits | mailbox index
     unsigned short* soff;    // float offset of its g-bar population
     unsigned short* rbox;    // index in the own mailbox of a received entry
     unsigned short* roff;    // float offset of its g-bar population
@@ -701,21 +701,16 @@ __device__ __forceinline__ void resident_body(S* __restrict__ state, const Geome
                 else collide_ace<T>(f, ph.c, m, omega_phi);
             }
             __syncthreads();   // every population of the round's rows is in registers
-            // the previous round's pushes into this round's first row (only the words that no push
-            // of this round writes: nothing orders the two)
-            if (rnd > 0) {
+            if (rnd > 0) {     // the previous round's pushes into this round's first row
                 constexpr int PLN[3] = {2, 5, 6};
                 const float* from = carry + ((rnd - 1) & 1) * ROWF;
                 float* to = pop + (1 + q) * ROWF;
-                const bool nsl = G.wall_x && B.strip == 0 && !(G.slip & 1);
-                const bool nsr = G.wall_x && B.strip == D.nstrip - 1 && !(G.slip & 2);
                 for (int k = tid; k < (PL / 3) * RW; k += NT) {
                     const int j = k / RW;
-                    const int a = j % 3 == 0 ? PLN[0] : j % 3 == 1 ? PLN[1] : PLN[2];
-                    const int p = (j >= 3 ? 9 : 0) + a;
-                    if (carry_fills(a, k % RW - 1, w, nsl, nsr))
-                        to[p * RW + k % RW] = from[p * RW + k % RW];
+                    const int p = (j >= 3 ? 9 : 0) + (j % 3 == 0 ? PLN[0] : j % 3 == 1 ? PLN[1] : PLN[2]);
+                    to[p * RW + k % RW] = from[p * RW + k % RW];
                 }
+                if (xwall && carry_meets_pushes(G.slip)) __syncthreads();
             }
             if (!live) continue;
             float* rC = pop + r * ROWF + cl + 1;

@@ -325,7 +325,9 @@ int lbm_check(lbm_ctx* ctx);
  * waits).  With enable = 2, runs of two or more steps of a context with the multi-step kernel
  * enabled (lbm_set_persistent) go to it as usual, but its waits for the neighbouring warps
  * between steps never succeed: after the first step every warp waits out its bound (two
- * seconds), records LBM_ERR_TIMEOUT and returns, with no copy in flight.  Nothing faults or
+ * seconds), records LBM_ERR_TIMEOUT and returns, with no copy in flight.  Runs that the resident
+ * kernel takes go to it, but its blocks send no messages: after the first step they wait out their
+ * bound (two seconds as well), record LBM_ERR_TIMEOUT and return.  Nothing faults or
  * hangs in either mode; the state of those steps is invalid, lbm_check reports LBM_ERR_TIMEOUT,
  * and re-initialising the state (lbm_init_fields*, lbm_set_populations, lbm_load_state) clears
  * the error.  enable = 0 (default) returns to normal waits; other values: LBM_ERR_ARG. */

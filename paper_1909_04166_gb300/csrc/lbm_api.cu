@@ -38,7 +38,7 @@ struct lbm_ctx {
     // graphs of 2 (k + 1) steps (k < kGraphSizes) from buffer 0 / 1, flow sign + / -
     cudaGraphExec_t graph[2][2][16];
     int use_graph;
-    int cut_first_wait;    // lbm_inject_timeout (1: first shared-memory wait, 2: neighbour wait)
+    int cut_first_wait;    // lbm_inject_timeout (1: first shared-memory wait, 2: neighbour waits)
     unsigned* prog;        // progress words of the multi-step kernel, one per warp
     int use_multi;         // lbm_set_persistent
     int multi_bps;         // resident blocks per SM of the multi-step kernel (0: not usable)
@@ -221,6 +221,18 @@ void* resident_lists(const lbm_ctx* c)
     return static_cast<char*>(c->box) + c->rplan.Z.box_bytes;
 }
 
+// Fresh mailboxes and exchange lists for the plan.
+cudaError_t prepare(lbm_ctx* c)
+{
+    c->rtag = 0;
+    return with_variant(c->P.precision, c->variant, [&](auto r, auto s, auto v) {
+        if constexpr (std::is_same<decltype(r), float>::value)
+            return prepare_resident<decltype(s), decltype(v)::value>(c->G, c->rplan, c->box,
+                                                                     resident_lists(c), c->st);
+        else return cudaErrorInvalidValue;
+    });
+}
+
 // Other contexts may run beside this one: it has a stream of its own (work on the default stream is
 // in one order).
 bool shares(const lbm_ctx* c)
@@ -235,7 +247,7 @@ bool shares(const lbm_ctx* c)
 // fastest form of a grid by itself (lbm_resident.cu has the times).
 bool resident_takes(lbm_ctx* c, long long run)
 {
-    if (!c->use_resident || !c->use_graph || c->checked || c->cut_first_wait ||
+    if (!c->use_resident || !c->use_graph || c->checked || c->cut_first_wait == 1 ||
         c->resident_state < 0 || run < kResidentMinSteps)
         return false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -260,13 +272,7 @@ bool resident_takes(lbm_ctx* c, long long run)
             c->box = nullptr;
             return false;
         }
-        const cudaError_t e = with_variant(c->P.precision, c->variant, [&](auto r, auto s, auto v) {
-            if constexpr (std::is_same<decltype(r), float>::value)
-                return prepare_resident<decltype(s), decltype(v)::value>(
-                    c->G, c->rplan, c->box, resident_lists(c), c->st);
-            else return cudaErrorInvalidValue;
-        });
-        if (e != cudaSuccess) return false;
+        if (prepare(c) != cudaSuccess) return false;
         c->resident_state = 1;
     }
     return true;
@@ -274,15 +280,19 @@ bool resident_takes(lbm_ctx* c, long long run)
 
 cudaError_t launch_resident_run(lbm_ctx* c, int nsteps, int sign)
 {
+    const bool mute = c->cut_first_wait == 2;   // lbm_inject_timeout: nobody sends
+    cudaError_t e = mute ? mute_resident(c->rplan, resident_lists(c), c->st) : cudaSuccess;
+    if (e != cudaSuccess) return e;
     const unsigned tag0 = c->rtag;
     c->rtag += (unsigned)nsteps;
-    return with_variant(c->P.precision, c->variant, [&](auto r, auto s, auto v) {
+    e = with_variant(c->P.precision, c->variant, [&](auto r, auto s, auto v) {
         if constexpr (std::is_same<decltype(r), float>::value)
             return launch_resident<decltype(s), decltype(v)::value>(
                 cur_state(c), c->G, c->Kf, c->rplan, nsteps, sign ? sign : 1, tag0, c->box,
                 resident_lists(c), c->err, c->st);
         else return cudaErrorInvalidValue;
     });
+    return mute && e == cudaSuccess ? prepare(c) : e;
 }
 
 void drop_graphs(lbm_ctx* c)
@@ -821,7 +831,6 @@ int lbm_set_resident(lbm_ctx* c, int32_t enable)
         if (e != cudaSuccess) return cuda_fail(c, e);
         cudaFree(c->box);
         c->box = nullptr;
-        c->rtag = 0;
         c->resident_state = 0;
     }
     return LBM_OK;

@@ -1087,6 +1087,12 @@ cudaError_t prepare_resident(const Geometry& G, const ResidentPlan& P, void* box
     return cudaGetLastError();
 }
 
+cudaError_t mute_resident(const ResidentPlan& P, void* lists, cudaStream_t st)
+{
+    const size_t pitch = (2 + list_words(P.Z.hmax, P.Z.tab)) * sizeof(int);   // a block's; its sends first
+    return cudaMemset2DAsync(lists, pitch, 0, sizeof(int), P.Z.nblocks, st);
+}
+
 template <typename S, int V>
 cudaError_t launch_resident(void* state, const Geometry& G, const Consts<float>& K,
                             const ResidentPlan& P, int nsteps, int flow_sign, unsigned tag0,

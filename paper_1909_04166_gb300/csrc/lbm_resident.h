@@ -74,6 +74,10 @@ cudaError_t launch_resident(void* state, const Geometry&, const Consts<float>&,
                             const ResidentPlan&, int nsteps, int flow_sign, unsigned tag0,
                             void* box, void* lists, int* err, cudaStream_t);
 
+// Empty the send lists, so that the waits of the next launch run out (a test of the way out), after
+// which the mailboxes and lists have to be prepared again.
+cudaError_t mute_resident(const ResidentPlan&, void* lists, cudaStream_t);
+
 // The same for a batch, one launch per wave, the wave of the most blocks first; false where a case
 // does not fit.  *step_us: what a step of all waves takes by the
 // planner's model.  The waves of a batch may share one set of mailboxes (zeroed by the caller), with tags that continue from launch

@@ -339,8 +339,8 @@ def lbm_check(ctx) -> None:
 
 def lbm_inject_timeout(ctx, enable) -> None:
     """Test hook of the failure path: 1, the first bounded wait of every warp of a step gives
-    up at once; 2, the multi-step kernel's waits for neighbouring warps never succeed (both
-    report LBM_ERR_TIMEOUT; nothing faults or hangs)."""
+    up at once; 2, the multi-step kernel's waits for neighbouring warps and the resident kernel's
+    for neighbouring blocks never succeed (all report LBM_ERR_TIMEOUT; nothing faults or hangs)."""
     _check(lib().lbm_inject_timeout(ctx, int(enable)), "lbm_inject_timeout")
 
 

@@ -325,3 +325,30 @@ def test_a_grid_that_shares_the_device_better_in_the_other_forms():
         lbm.lbm_set_resident(sim.ctx, 2)
         assert lbm.lbm_get_run_path(sim.ctx, 40)[0] == lbm.LBM_PATH_RESIDENT
         assert lbm.lbm_get_run_path(default.ctx, 40)[0] == lbm.LBM_PATH_RESIDENT
+
+
+@pytest.mark.parametrize("form", ["fp32", "half rows", "bf16", "flow"])
+def test_waits_for_messages_run_out_and_are_reported(form):
+    """The waits for the neighbouring blocks are bounded: where no messages come (none is sent), every
+    block gives up after its first step and the run reports LBM_ERR_TIMEOUT; initialising the state
+    again clears it, and the same mailboxes then serve a run like a fresh context's."""
+    case = (W.shear_circle(L0=130, u0=0.03) if form == "flow" else
+            W.random_drop(70, 60, seed=7, wall_y=1, rho_ratio=100.0) if form == "half rows" else
+            W.random_drop(200, 700, seed=7, wall_x=1, rho_ratio=100.0))
+    precision = "bf16" if form == "bf16" else "fp32"
+    with lbm.Simulation(case, precision=precision) as a, \
+            lbm.Simulation(case, precision=precision) as fresh:
+        a.init_case().step(20)
+        lbm.lbm_check(a.ctx)
+        lbm.lbm_inject_timeout(a.ctx, 2)
+        assert lbm.lbm_get_run_path(a.ctx, 40)[0] == lbm.LBM_PATH_RESIDENT
+        a.step(40)
+        for read in (lambda: lbm.lbm_check(a.ctx), a.fields, a.save_state):
+            with pytest.raises(lbm.LbmError) as e:
+                read()
+            assert e.value.status == lbm.LBM_ERR_TIMEOUT
+        lbm.lbm_inject_timeout(a.ctx, 0)
+        a.init_case().step(37)
+        lbm.lbm_check(a.ctx)
+        fresh.init_case().step(37)
+        assert np.array_equal(a.save_state()[0], fresh.save_state()[0])

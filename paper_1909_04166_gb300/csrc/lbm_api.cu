@@ -106,10 +106,11 @@ constexpr int kSegRows = 16;
 // the rows of a segment, about kDpRow instructions each, and the sums of the two rows around it
 // (kDpSeg); the fewer warps share the SM, the more of their other latencies shows (kDpFew).  With
 // one-warp blocks the scheduler spreads the warps evenly; warps beyond the resident ones wait for a
-// second wave.  The shortest such time over the segment heights up to kDpMaxRows decides (one GB300, us a step with the 365
-// instructions a row that the update took before, the former whole-wave rule in 4-warp blocks against
-// this one: 64 x 64 18.0 / 16.5, 256 x 256 57.8 / 50.4, 512 x 256 123 / 94, 700 x 450 238 / 218,
-// 600 x 300 162 / 138).
+// second wave.  The shortest such time over the segment heights up to kDpMaxRows decides (one GB300,
+// us a step, the former whole-wave rule in 4-warp blocks against this one, both with the 365
+// instructions a row that the update took before: 64 x 64 18.0 / 16.5, 256 x 256 57.8 / 50.4, 512 x
+// 256 123 / 94, 700 x 450 238 / 218, 600 x 300 162 / 138; rule and update as they were against both as
+// they are: 256 x 1024 201 / 148, 512 x 256 123 / 72, 2048 x 1024 1468 / 1043, 65536 x 8 422 / 285).
 constexpr double kDpSm = 19, kDpWarp = 64, kDpRow = 270, kDpSeg = 50, kDpFew = 0.3;
 constexpr int kDpMaxRows = 24;
 

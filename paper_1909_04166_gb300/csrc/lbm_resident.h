@@ -79,9 +79,9 @@ cudaError_t launch_resident(void* state, const Geometry&, const Consts<float>&,
 cudaError_t mute_resident(const ResidentPlan&, void* lists, cudaStream_t);
 
 // The same for a batch, one launch per wave, the wave of the most blocks first; false where a case
-// does not fit.  *step_us: what a step of all waves takes by the
-// planner's model.  The waves of a batch may share one set of mailboxes (zeroed by the caller), with tags that continue from launch
-// to launch; case_of[b] is the index into `cases` of block b of the wave.
+// does not fit.  *step_us: what a step of all waves takes by the planner's model.  The waves of a batch
+// may share one set of mailboxes (zeroed by the caller), with tags that continue from launch to
+// launch; case_of[b] is the index into `cases` of block b of the wave.
 template <typename S, int V>
 bool resident_batch_plan(const Geometry*, int ncases, int nsm, std::vector<ResidentWave>*,
                          double* step_us);

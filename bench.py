@@ -90,19 +90,20 @@ def kernel_source_hash() -> str:
 # DRAM traffic per step of the step kernels from ncu captures (dram__bytes_read.sum +
 # dram__bytes_write.sum), keyed by the hash of the kernel sources they were taken on, the
 # workload, the precision and the launch form ("step": one launch per step, the mean of three
-# consecutive launches; "multi": one launch of the multi-step kernel divided by its steps).
+# consecutive launches; "multi": one launch of the multi-step kernel divided by its steps;
+# "resident": not per step but per launch of the resident kernel, for the batch per run of all waves).
 # Caches are not flushed between launches, as in the timed run; the bench line reports the
 # bytes of one of its launches.
 NCU_TRAFFIC = {
     # multi-step kernel (FP32, the default for runs on the 2048 x 1024 impact), sources
-    # 52b32e0d7565347e: one launch of 32 steps read 3711.62 MB + wrote 4843.53 MB; per step
-    ("52b32e0d7565347e", "impact", "fp32", "multi"): 267_348_568,
+    # 8c6e52da611e5d13: one launch of 32 steps read 3697.21 MB + wrote 4844.83 MB; per step
+    ("8c6e52da611e5d13", "impact", "fp32", "multi"): 266_938_800,
     # FP16-storage step kernel (graph replays, one launch per step) on the same grid and
-    # sources: read 48.05 MB + write 92.33 MB per launch
-    ("52b32e0d7565347e", "impact", "fp16", "step"): 140_380_757,
-    # batched step of the 512-case ensemble (autotuned: 8 rows per task, 128-thread blocks), same
-    # sources: read 839.67 MB + write 760.12 MB per launch
-    ("52b32e0d7565347e", "ensemble", "fp32", "step"): 1_599_791_019,
+    # sources: read 47.59 MB + write 92.36 MB per launch
+    ("8c6e52da611e5d13", "impact", "fp16", "step"): 139_947_691,
+    # resident waves of the 512-case ensemble (38 launches for a run), same sources: read 914.39 MB +
+    # write 806.57 MB per run
+    ("8c6e52da611e5d13", "ensemble", "fp32", "resident"): 1_720_964_864,
 }
 
 
@@ -291,11 +292,11 @@ def run_ours(args):
     }.get(path, ("step", "cmlbm::step_kernel" + narrow,
                  "graph replays of one step-kernel launch per step"))
     key = (hsh, args.workload, args.precision, form)
-    if key in NCU_TRAFFIC:   # DRAM bytes per step, for this launch's steps
-        traffic = int(round(NCU_TRAFFIC[key] * steps_per_launch))
     # the resident kernel reads and writes the state once a launch: no share of the HBM rate then
     # says how near the kernel is to its bound
     resident = path == lbm.LBM_PATH_RESIDENT
+    if key in NCU_TRAFFIC:   # DRAM bytes per step (for this launch's steps); resident: per launch
+        traffic = int(round(NCU_TRAFFIC[key] * (1 if resident else steps_per_launch)))
     value = job_mlups(ws, N, K, ms_max)
     line = {
         "metric": METRIC,

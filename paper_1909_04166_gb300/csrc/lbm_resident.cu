@@ -708,9 +708,13 @@ __device__ __forceinline__ void resident_body(S* __restrict__ state, const Geome
                 for (int k = tid; k < (PL / 3) * RW; k += NT) {
                     const int j = k / RW;
                     const int p = (j >= 3 ? 9 : 0) + (j % 3 == 0 ? PLN[0] : j % 3 == 1 ? PLN[1] : PLN[2]);
+                    if (SHEAR && !carry_fills(p, k % RW - 1, w,
+                                              G.wall_x && B.strip == 0 && !(G.slip & 1),
+                                              G.wall_x && B.strip == D.nstrip - 1 && !(G.slip & 2)))
+                        continue;
                     to[p * RW + k % RW] = from[p * RW + k % RW];
                 }
-                if (xwall && carry_meets_pushes(G.slip)) __syncthreads();
+                if (!SHEAR && xwall && carry_meets_pushes(G.slip)) __syncthreads();
             }
             if (!live) continue;
             float* rC = pop + r * ROWF + cl + 1;

@@ -20,13 +20,20 @@ constexpr int kResidentWarps = 16;   // warps of a block; one block per SM
 // it, all columns of which the next round, whose first row that is, copies into place and then pushes.
 // Two words of such a row come from nowhere in the round before: plane 5 of the first column beside a
 // no-slip left side and plane 6 of the last one beside a no-slip right side, which the row's own node
-// bounces back there in the round of the copy.  The copy, which has nothing valid for them, then has to
-// be over first: a barrier in blocks at a walled side of a grid with a no-slip one (slip: the free-slip
-// sides, bit 0 left, bit 1 right).  Elsewhere, a free-slip side mirroring populations 6 and 5 of the row
-// below into the same words, copy and pushes write different words.  (Leaving the two words out of the
-// copy instead came out at 5.76 us a step at 256 x 1024, this at 5.70, where the whole copy without a
-// barrier took 5.69.)
+// bounces back there in the round of the copy.  (A free-slip side mirrors populations 6 and 5 of the
+// row below into the same words; they then come from the round before, and copy and pushes write
+// different words, as they do everywhere else.)  The copy has nothing valid for the two: either it is
+// over before the pushes, by a barrier in blocks at a walled side of a grid with a no-slip one (slip: the
+// free-slip sides, bit 0 left, bit 1 right), or it leaves them out.  The two lattices take the barrier,
+// the interface lattice alone the shorter copy, which each came out faster, through the registers of
+// the whole loop also on grids without such sides: us a step at 256 x 1024 5.70 against 5.76, imposed
+// flow 800 x 800 8.04 against 7.86 (the whole copy without a barrier: 5.69 and 7.94).
 CMLBM_RULE bool carry_meets_pushes(int slip) { return (slip & 3) != 3; }
+CMLBM_RULE bool carry_fills(int plane, int column, int width, bool noslip_left, bool noslip_right)
+{
+    return !(noslip_left && plane == 5 && column == 0) &&
+           !(noslip_right && plane == 6 && column == width - 1);
+}
 
 // ---- plans ----------------------------------------------------------------------------------
 struct GridSize {

@@ -41,34 +41,49 @@ def landings(row, width, sides, top=None, wall=0):
 
 
 @pytest.mark.parametrize("width", [1, 2, 37, 63, 64])
-def test_a_barrier_stands_where_the_carry_copy_meets_pushes(tmp_path, width):
-    """A round copies planes 2, 5 and 6 of its first row from the carry and pushes its own rows with
-    nothing between them but where carry_meets_pushes says so: there only may both write a word.  The
-    words that no push of the round before filled are overwritten by those pushes, or by a message."""
-    (out,) = compiled(tmp_path, """
-int main() { for (int slip = 0; slip < 4; ++slip) std::printf("%d ", (int)carry_meets_pushes(slip)); }""")
+def test_carry_copy_and_pushes_write_different_words_or_have_a_barrier(tmp_path, width):
+    """A round copies planes 2, 5 and 6 of its first row from the carry and pushes its own rows.  Both
+    write a word only where carry_meets_pushes asks for a barrier between them; the shorter copy
+    (carry_fills) never does, and leaves out nothing that the round before pushed.  What else the
+    copies bring is overwritten by those pushes, or by a message."""
+    out = compiled(tmp_path, f"""
+int main()
+{{
+    for (int slip = 0; slip < 4; ++slip) std::printf("%d ", (int)carry_meets_pushes(slip));
+    std::printf("\\n");
+    for (int l = 0; l < 2; ++l) for (int r = 0; r < 2; ++r)
+        for (int p = 2; p < 7; ++p) for (int c = -1; c <= {width}; ++c)
+            if (p == 2 || p > 4) std::printf("%d %d %d %d %d\\n", l, r, p, c,
+                                             (int)carry_fills(p, c, {width}, l, r));
+}}""")
+    barrier = [t == "1" for t in out[0]]
     copied = {(c, p) for c in range(-1, width + 1) for p in (2, 5, 6)}
+    shorter = {}
+    for l, r, p, c, on in (map(int, t) for t in out[1:]):
+        shorter.setdefault((l, r), set()).update({(c, p)} if on else set())
     first = 17
     met = set()
     for left in (0, 1, 2):
         for right in (0, 1, 2):
             slip = (left == 2) + 2 * (right == 2)
+            few = shorter[left == 1, right == 1]
             for top, wall in ((None, 0), (first, 1), (first, 2), (first + 1, 1), (first + 1, 2)):
                 sides = (left, right)
                 before = {(c, a) for r, c, a in landings(first - 1, width, sides) if r == first}
                 rows = [first] if top == first else [first, first + 1]
                 during = {(c, a) for row in rows
                           for r, c, a in landings(row, width, sides, top, wall) if r == first}
-                assert before <= copied and not before & during
+                assert before <= few <= copied and not before & during
+                assert not few & during, (sides, top, wall)
                 if copied & during:   # (a block at a wall: xwall)
-                    assert 1 in sides and out[slip] == "1", (sides, top, wall)
+                    assert 1 in sides and barrier[slip], (sides, top, wall)
                     met.add(sides)
                 for c, a in copied - before - during:   # from beyond the strip, or a ghost node
                     assert not 0 <= c < width or not 0 <= c - EX[a] < width
                     assert not (c == 0 and left == 1 and a == 5)
                     assert not (c == width - 1 and right == 1 and a == 6)
     assert met == {(l, r) for l in (0, 1, 2) for r in (0, 1, 2) if 1 in (l, r)}
-    assert out[3] == "0"      # and no barrier between two free-slip sides
+    assert not barrier[3]     # and no barrier between two free-slip sides
 
 
 PLAN = """

@@ -96,14 +96,14 @@ def kernel_source_hash() -> str:
 # bytes of one of its launches.
 NCU_TRAFFIC = {
     # multi-step kernel (FP32, the default for runs on the 2048 x 1024 impact), sources
-    # 8c6e52da611e5d13: one launch of 32 steps read 3697.21 MB + wrote 4844.83 MB; per step
-    ("8c6e52da611e5d13", "impact", "fp32", "multi"): 266_938_800,
+    # a8fb514c5190d931: one launch of 32 steps read 3534.71 MB + wrote 4844.36 MB; per step
+    ("a8fb514c5190d931", "impact", "fp32", "multi"): 261_845_696,
     # FP16-storage step kernel (graph replays, one launch per step) on the same grid and
-    # sources: read 47.59 MB + write 92.36 MB per launch
-    ("8c6e52da611e5d13", "impact", "fp16", "step"): 139_947_691,
-    # resident waves of the 512-case ensemble (38 launches for a run), same sources: read 914.39 MB +
-    # write 806.57 MB per run
-    ("8c6e52da611e5d13", "ensemble", "fp32", "resident"): 1_720_964_864,
+    # sources: read 47.60 MB + write 92.36 MB per launch
+    ("a8fb514c5190d931", "impact", "fp16", "step"): 139_960_832,
+    # resident waves of the 512-case ensemble (38 launches for a run), same sources: read 914.37 MB +
+    # write 806.73 MB per run
+    ("a8fb514c5190d931", "ensemble", "fp32", "resident"): 1_721_101_056,
 }
 
 
